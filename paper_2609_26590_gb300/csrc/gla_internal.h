@@ -82,6 +82,9 @@ bool tc_gate_supported(const Problem &p, int rank);
 // problem's g pointer is not used).
 cudaError_t launch_tc_gate(const Problem &p, const GateSource &gs, cudaStream_t stream, Ran *ran = nullptr);
 
+// SMs of the current device, looked up once per device.
+cudaError_t sm_count(int *n_sm);
+
 // Device status word of the current device (set by bounded device waits).
 cudaError_t read_and_clear_device_status(unsigned int *status);
 

@@ -624,20 +624,18 @@ template <int DKM, typename E, bool VEC>
 cudaError_t launch_shape(const Problem &p, cudaStream_t stream) {
     using Sh = SimtShape<DKM>;
     static std::atomic<unsigned long long> set_on_devices(0);
-    static std::atomic<int> sms[64] = {};
     auto kernel = gla_simt_kernel<DKM, E, VEC>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int n_sm = sms[dev & 63].load(std::memory_order_relaxed);
+    int n_sm = 0;
+    if ((e = sm_count(&n_sm)) != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
-    if (!(set_on_devices.load(std::memory_order_acquire) & bit)) {
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::bytes)) != cudaSuccess ||
+    if (!(set_on_devices.load(std::memory_order_relaxed) & bit)) {
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::bytes)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
             return e;
-        sms[dev & 63].store(n_sm, std::memory_order_relaxed);
-        set_on_devices.fetch_or(bit, std::memory_order_release);
+        set_on_devices.fetch_or(bit);
     }
     SimtParams sp;
     sp.p = p;

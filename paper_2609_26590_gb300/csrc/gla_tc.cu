@@ -1610,23 +1610,6 @@ unsigned long long next_epoch() {
     return ctr.fetch_add(2ull);  // odd, so never 0
 }
 
-cudaError_t sm_count(int *n_sm) {  // cached per device
-    static std::atomic<int> cache[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) {
-        const int v = cache[dev].load(std::memory_order_relaxed);
-        if (v > 0) {
-            *n_sm = v;
-            return cudaSuccess;
-        }
-    }
-    e = cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) cache[dev].store(*n_sm, std::memory_order_relaxed);
-    return e;
-}
-
 // Key channels and value columns are processed in 64-wide halves and slices; a
 // narrower last one is zero-padded by the TMA loads (boxes past the tensor's row).
 int pad64(int d) { return (d + 63) / 64 * 64; }
@@ -1696,6 +1679,23 @@ size_t summary_bytes(const Problem &p, int nseg) {
 }
 
 }  // namespace
+
+cudaError_t sm_count(int *n_sm) {  // cached per device
+    static std::atomic<int> cache[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) {
+        const int v = cache[dev].load(std::memory_order_relaxed);
+        if (v > 0) {
+            *n_sm = v;
+            return cudaSuccess;
+        }
+    }
+    e = cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) cache[dev].store(*n_sm, std::memory_order_relaxed);
+    return e;
+}
 
 int tc_chunk_boxes(int order, int T, int grid_h, int grid_w, int c, int *boxes, int cap) {
     int n = 0;
