@@ -30,6 +30,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "f32x2.cuh"
 #include "fastdiv.cuh"
 #include "gla_internal.h"
 #include "tc_ptx.cuh"
@@ -61,33 +62,6 @@ struct SwParams {
     uint32_t vbytes, gbytes;  // bytes of the value box and of the gate box
 };
 
-// Two fp32 values in one 64-bit register, and the packed IEEE operations on them.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-    return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 // SiLU(z) = z / (1 + e^{-z}) of a pair, by the hardware's 2^x and 1/x.  Flushing their subnormal
 // results changes nothing: 1 + e is 1 there, and z / (1 + e) is below 2^-120 where 1/(1 + e) is.
 __device__ __forceinline__ f2 silu2(f2 z) {
