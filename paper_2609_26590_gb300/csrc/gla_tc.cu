@@ -1020,11 +1020,10 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const float am1 = ref[lane + 32] * kLog2e, al1 = ref[kD + lane + 32] * kLog2e;
                 float m = fmaxf(fmaxf(-am0, am0 - al0), fmaxf(-am1, am1 - al1));
                 if (!(m <= 3.0e38f)) m = 3.0e38f;  // NaN / inf gates: exact path
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+                // (m >= 0 for log gates <= 0, so its bits order like the values.)  One redux instead of five
+                // shuffles and maxima: every warp waits for this, 1.13x at Dk = Dv = 128 and 1.04x at
+                // B = 32, H = 12, 40 x 40 on a GB300
+                m = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(m)));
                 mode = m <= kMaxRefF16 ? kModeF16 : (m <= kMaxRefTF32 ? kModeTF32 : kModeExact);
                 if (tg < 32) {
                     ref[2 * kD + lane] = ex2(am0);
@@ -1034,6 +1033,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     decay_s[sl * kD + lane] = ex2(al0);
                     decay_s[sl * kD + lane + 32] = ex2(al1);
                     if (tg == 0) mode_s[sl] = mode;
+                    __syncwarp();
+                    // constants and mode of chunk c -> epi, written by this warp
+                    if (tg == 0 && mode != kModeExact) mbar_arrive(&bars[BAR_REFS + sl]);
                 }
             }
             uint8_t *tq = st + kQ, *tk = st + kK, *tgt = st + kG;
@@ -1093,11 +1095,15 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             }
             fence_proxy_async_smem();
             tc_fence_before();
-            if (named_barrier_or(bar_id, 128, opfail)) {
-                record_timeout(abort_flag);
-                break;
+            // (no group barrier: every thread rewrote only what it read, and each warp signals its own rows;
+            // an exact chunk's decays are the whole group's)
+            if (mode == kModeExact) {
+                if (named_barrier_or(bar_id, 128, opfail)) {
+                    record_timeout(abort_flag);
+                    break;
+                }
+                if (tg == 0) mbar_arrive(&bars[BAR_REFS + sl]);  // constants and mode of chunk c -> epi
             }
-            if (tg == 0) mbar_arrive(&bars[BAR_REFS + sl]);  // constants and mode of chunk c -> epi
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_PURDY + bb]);  // operands in smem, A(c) read
             if (kSum) continue;  // no scores
@@ -1108,10 +1114,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 if (c >= 2) ofail = !gen_out(c - 2);
             }
             // ---- masked scores of chunk c over its gate tile (consumed by A(c) long ago)
+            // (a warp that gives up here skips the rest of the chunk; the group leaves together at
+            // the barrier of its next one)
             const bool pfail = ofail || !mbar_wait(&bars[BAR_PFULL + bb], ph, abort_flag, kWaitLimitNs);
-            if (named_barrier_or(bar_id, 128, pfail)) {
-                record_timeout(abort_flag);
-                break;
+            if (__any_sync(0xffffffffu, pfail)) {
+                if (lane == 0) record_timeout(abort_flag);
+                continue;
             }
             if (mode != kModeExact) {
                 tc_fence_after();
