@@ -435,6 +435,51 @@ __device__ __forceinline__ int walk_token(int order, int T, const FastDiv &gh, i
     return (w - x * gh.d) * grid_w + x;
 }
 
+// Stores a row's 32 output columns (col0 ..., four 16-byte pieces) of token t per lane, lanes l and
+// l ^ 1 holding two rows.  Stored as they are, every instruction writes 16 bytes into each of 32
+// sectors; the pair first swaps pieces so that its two lanes write 32 consecutive bytes of one row
+// (GB300, graph replays: 6,400 tokens 170 -> 155 us, 704^2 images with Dk = 32 42 -> 39 us, B = 32,
+// H = 12, 40 x 40 87 -> 84 us; a 4 x 4 transpose to 64 bytes costs more instructions than it gives).
+// With two key halves and split sequences the epi has no registers left for it (252 us against 255 at
+// 128 x 128; whole sequences 198 -> 185 us).
+template <typename E, bool PAIR>
+__device__ __forceinline__ void store_row(const TcParams &p, const uint32_t (&ow)[16], int b, int h, int t, int col0) {
+    if constexpr (PAIR) {
+        uint4 pc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) pc[q] = make_uint4(ow[4 * q], ow[4 * q + 1], ow[4 * q + 2], ow[4 * q + 3]);
+        const bool odd = threadIdx.x & 1;
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+            // the even lane gives its odd pieces for the odd lane's even ones
+            uint4 s = odd ? pc[q] : pc[q + 1];
+            s.x = __shfl_xor_sync(0xffffffffu, s.x, 1);
+            s.y = __shfl_xor_sync(0xffffffffu, s.y, 1);
+            s.z = __shfl_xor_sync(0xffffffffu, s.z, 1);
+            s.w = __shfl_xor_sync(0xffffffffu, s.w, 1);
+            if (odd) pc[q] = s;
+            else pc[q + 1] = s;
+        }
+        // now pc[q] is the even lane's row and pc[q + 1] the odd lane's, at piece q + odd
+        const int other = __shfl_xor_sync(0xffffffffu, t, 1);
+        const int t0 = odd ? other : t, t1 = odd ? t : other;
+        const int col = col0 + 8 * odd, ld = p.H * p.Dv;
+        E *base = static_cast<E *>(p.out) + ((size_t)b * p.T * p.H + h) * p.Dv + col;
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+            if (col + 8 * q < p.Dv) {  // (columns past Dv and rows outside the sequence stay behind)
+                if (t0 >= 0) *reinterpret_cast<uint4 *>(base + (size_t)t0 * ld + 8 * q) = pc[q];
+                if (t1 >= 0) *reinterpret_cast<uint4 *>(base + (size_t)t1 * ld + 8 * q) = pc[q + 1];
+            }
+        }
+    } else if (t >= 0) {
+        uint4 *dst = reinterpret_cast<uint4 *>(static_cast<E *>(p.out) + (((size_t)b * p.T + t) * p.H + h) * p.Dv + col0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (col0 + 8 * q < p.Dv) dst[q] = make_uint4(ow[4 * q], ow[4 * q + 1], ow[4 * q + 2], ow[4 * q + 3]);
+    }
+}
+
 // Exact scores for one chunk (extreme or non-finite log-decays): serial prefix
 // of the clamped gates, P[rho][sigma] = sum_i q k 2^{a_r,i - a_j,i} (j <= r) by
 // CUDA cores, Qtil = q 2^{a}, Kbar = k 2^{a_last - a}, and the chunk decay.
@@ -588,6 +633,13 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     // which takes that work off the epi's serial per-chunk chain.  The host selects it where
     // that was measured faster (fp16 launches of at most one wave); elsewhere the epi stores.
     constexpr bool kGenOut = GENOUT && NH == 1 && !kSum;
+    // The SM's instruction cache is shared by all roles, and the hot loops do not fit it (ncu: 9 % of
+    // its requests miss on B = 32, H = 12, 40 x 40, 35 % with the gate producer).  The fp16 operand
+    // build therefore runs as a loop over two halves of a thread's channels, each read from TMEM when
+    // its turn comes, where the epi stores the outputs (GB300, graph replays: 84.5 -> 82.3 us there,
+    // Dk = Dv = 128 188 -> 185 us); unrolled it is faster where the gen warps store them (6,400 tokens,
+    // tf32 scores: 155 us against 171).
+    constexpr bool kRollBuild = !kGenOut;
     const int N = p.n_chunks;   // chunks per sequence
     const int L = p.seg_len;    // chunks per unit
     constexpr int nh = NH;   // 64-channel key halves per chunk (Dk / 64)
@@ -801,8 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 }
                 const uint64_t dg = mndesc(slot0 + (ca % kSlots) * kSlotBytes + kG);
                 const uint32_t d = tmem + kColA + (ca & 1) * 64;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) mma_f16_ss_warp(d, dL + 2 * ks, dg + 128 * ks, idesc_a, ks > 0);
+                mma4_f16_ss_warp<2, 128>(d, dL, dg, idesc_a, 0);
                 mma_commit_warp(&bars[BAR_AFULL + (ca & 1)]);
             }
         } else if (warp == 14) {
@@ -822,16 +873,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     // summaries need no scores
                 } else if (mode == kModeF16) {
                     const uint64_t dq = kdesc(st + kQ), dk = kdesc(st + kK);
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) mma_f16_ss_warp(dp, dq + 2 * ks, dk + 2 * ks, idesc_p16, ks > 0);
+                    mma4_f16_ss_warp<2, 2>(dp, dq, dk, idesc_p16, 0);
                     mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
                 } else if (mode == kModeTF32) {
                     const uint64_t dqh = dqh0 + (c & 1) * (2 * kTile32 >> 4), dkh = dkh0 + (c & 1) * (2 * kTile32 >> 4);
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint32_t off = (ks >> 2) * 512 + (ks & 3) * 2;  // (8192 B, 32 B) >> 4
-                        mma_tf32_ss_warp(dp, dqh + off, dkh + off, idesc_p32, ks > 0);
-                    }
+                    mma4_tf32_ss_warp(dp, dqh, dkh, idesc_p32, 0);
+                    mma4_tf32_ss_warp(dp, dqh + 512, dkh + 512, idesc_p32, 1);  // (the second 32 columns: 8192 B >> 4)
                     mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
                 } else if (lane == 0) {
                     mbar_arrive(&bars[BAR_PFULL + (c & 1)]);  // exact scores are already in smem
@@ -840,10 +887,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 // U(c) = Kbar^T V (fp16 mode: K^^T V): the k tile read as the MN-major A
                 const uint64_t dk = mndesc(st + kK), dv = mndesc(st + kV);
                 const uint32_t du = tmem + kColU + (c & 1) * 64;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) mma_f16_ss_warp(du, dk + 128 * ks, dv + 128 * ks, idesc_u, ks > 0);
-                mma_commit_warp(&bars[BAR_UFULL + (c & 1)]);
-                mma_commit_warp(&bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
+                mma4_f16_ss_warp<128, 128>(du, dk, dv, idesc_u, 0);
+                mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
                 su = (su == kSlots - 1) ? 0 : su + 1;
             }
         } else if (!kSum) {
@@ -861,12 +906,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint64_t dpm = kdesc(st + kG), dv = mndesc(st + kV);
                 const uint32_t d = tmem + kColO + ((c / nh) & 1) * 64;
                 const uint32_t acc0 = (c % nh) != 0;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) mma_f16_ss_warp(d, dq + 2 * ks, ds + 128 * ks, idesc_o, acc0 | (ks > 0));
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) mma_f16_ss_warp(d, dpm + 2 * ks, dv + 128 * ks, idesc_o, 1);
-                mma_commit_warp(&bars[BAR_OFULL + (c & 1)]);
-                mma_commit_warp(&bars[BAR_EMPTY + so]);  // every product of the slot's chunk is done
+                mma4_f16_ss_warp<2, 128>(d, dq, ds, idesc_o, acc0);
+                mma4_f16_ss_warp<2, 128>(d, dpm, dv, idesc_o, 1);
+                mma_commit2_warp(&bars[BAR_OFULL + (c & 1)], &bars[BAR_EMPTY + so]);  // every product of the slot's chunk is done
                 so = (so == kSlots - 1) ? 0 : so + 1;
             }
         }
@@ -937,13 +979,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
 #pragma unroll
                 for (int j = 0; j < 16; ++j) ow[j] = Elem<E>::pack(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
             }
-            if (t >= 0) {  // the row's columns inside Dv (padded columns stay behind)
-                const int col0 = 64 * po.vb + ch0;
-                uint4 *dst = reinterpret_cast<uint4 *>(static_cast<E *>(p.out) + (((size_t)b * p.T + t) * p.H + h) * p.Dv + col0);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (col0 + 8 * q < p.Dv) dst[q] = make_uint4(ow[4 * q], ow[4 * q + 1], ow[4 * q + 2], ow[4 * q + 3]);
-            }
+            store_row<E, true>(p, ow, b, h, t, 64 * po.vb + ch0);
             return true;
         };
         int last_c = -1;  // the group's last chunk completed (its outputs are stored after the loop)
@@ -993,19 +1029,33 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             // normal range); the loads go first so that their latency hides behind the
             // operand build, the converted words are stored with the operands
             tc_fence_after();
-            uint32_t ar[32];
-            tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + bb * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&ar[0]));
-            tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + bb * 64 + 16, *reinterpret_cast<uint32_t(*)[16]>(&ar[16]));
-            tmem_ld_wait();
+            const uint32_t ta = tmem + lane_base + kColA + bb * 64;
             // references of chunk c: [0,64) raw A_mid, [64,128) raw A_last, [128,192) c1 = 2^{A_mid},
             // [192,256) c2 = 2^{A_last - A_mid}
             float *ref = reinterpret_cast<float *>(smem + kOffRef) + sl * kRefFloats;
-            if (!fail && (row == rho_mid || row == rho_last)) {
-                float *dst = ref + (row == rho_mid ? 0 : kD) + ch0;
+            auto write_refs = [&](const uint32_t (&a)[32]) {
+                if (!fail && (row == rho_mid || row == rho_last)) {
+                    float *dst = ref + (row == rho_mid ? 0 : kD) + ch0;
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    reinterpret_cast<float4 *>(dst)[q] = make_float4(__uint_as_float(ar[4 * q]), __uint_as_float(ar[4 * q + 1]),
-                                                                     __uint_as_float(ar[4 * q + 2]), __uint_as_float(ar[4 * q + 3]));
+                    for (int q = 0; q < 8; ++q)
+                        reinterpret_cast<float4 *>(dst)[q] = make_float4(__uint_as_float(a[4 * q]), __uint_as_float(a[4 * q + 1]),
+                                                                         __uint_as_float(a[4 * q + 2]), __uint_as_float(a[4 * q + 3]));
+                }
+            };
+            uint32_t ar[32];  // the thread's log-decays (unused with kRollBuild)
+            if constexpr (kRollBuild) {
+                if (q4 == rho_mid >> 4 || q4 == rho_last >> 4) {  // (the warps of the reference rows)
+                    uint32_t a[32];
+                    tmem_ld_16x32bx2_x16(ta + 0, *reinterpret_cast<uint32_t(*)[16]>(&a[0]));
+                    tmem_ld_16x32bx2_x16(ta + 16, *reinterpret_cast<uint32_t(*)[16]>(&a[16]));
+                    tmem_ld_wait();
+                    write_refs(a);
+                }
+            } else {
+                tmem_ld_16x32bx2_x16(ta + 0, *reinterpret_cast<uint32_t(*)[16]>(&ar[0]));
+                tmem_ld_16x32bx2_x16(ta + 16, *reinterpret_cast<uint32_t(*)[16]>(&ar[16]));
+                tmem_ld_wait();
+                write_refs(ar);
             }
             tc_fence_before();
             if (named_barrier_or(bar_id, 128, fail || *abort_flag != 0u)) {  // the group gives up together
@@ -1046,9 +1096,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 opfail = named_barrier_or(bar_id, 128, false);
             }
             if (mode == kModeF16) {
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    const int cl = ch0 + 8 * g8;
+                // the operands of channels cl .. cl + 7, whose log-decays are a[i0 ...]
+                auto build8 = [&](const auto &a, int i0, int cl) {
                     const ulonglong2 am0 = *reinterpret_cast<const ulonglong2 *>(ref + cl);  // raw A_mid of 8 channels
                     const ulonglong2 am1 = *reinterpret_cast<const ulonglong2 *>(ref + cl + 4);
                     const f2 am[4] = {am0.x, am0.y, am1.x, am1.y};
@@ -1062,7 +1111,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     uint32_t qo[4], ko[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const f2 x = fma2(pack2(ar[8 * g8 + 2 * e], ar[8 * g8 + 2 * e + 1]), pack2(kLog2e, kLog2e),
+                        const f2 x = fma2(pack2(a[i0 + 2 * e], a[i0 + 2 * e + 1]), pack2(kLog2e, kLog2e),
                                           mul2(am[e], pack2(-kLog2e, -kLog2e)));
                         qo[e] = h2bits(mul2(Elem<E>::unpack_pair(qa[e]), ex2_pair(x)));
                         ko[e] = h2bits(mul2(Elem<E>::unpack_pair(ka[e]), ex2_neg_pair(x)));
@@ -1070,10 +1119,23 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     // Q^ over q, K^ over k (each thread rewrites exactly what it read)
                     if (!kSum) *reinterpret_cast<uint4 *>(tq + o16) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
                     *reinterpret_cast<uint4 *>(tk + o16) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
+                };
+                if constexpr (kRollBuild) {
+#pragma unroll 1
+                    for (int hf = 0; hf < 2; ++hf) {
+                        uint32_t a[16];
+                        tmem_ld_16x32bx2_x16(ta + 16 * hf, a);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int g8 = 0; g8 < 2; ++g8) build8(a, 8 * g8, ch0 + 16 * hf + 8 * g8);
+                    }
+                } else {
+#pragma unroll
+                    for (int g8 = 0; g8 < 4; ++g8) build8(ar, 8 * g8, ch0 + 8 * g8);
                 }
             } else if (!opfail) {
                 if (mode == kModeTF32)
-                    tf32_operands<E>(tq, tk, smem + kOffOp + gw * 2 * kTile32, ref, tmem + lane_base + kColA + bb * 64, row, ch0);
+                    tf32_operands<E>(tq, tk, smem + kOffOp + gw * 2 * kTile32, ref, ta, row, ch0);
                 else
                     exact_chunk<E, GE>(tq, tk, tgt, reinterpret_cast<float *>(smem + kOffOp + gw * 2 * kTile32), decay_s + sl * kD, rev, tg,
                                    bar_id);
@@ -1155,7 +1217,6 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         const int row = 16 * q4 + (lane & 15);   // channel i for U / S, token rho for O
         const int ch0 = 32 * hc;
         const uint32_t lane_base = static_cast<uint32_t>(32 * q4) << 16;
-        E *out = static_cast<E *>(p.out);
         f2 S[16], So[NH == 2 ? 16 : 1];  // packed pairs of columns
 #pragma unroll
         for (int j = 0; j < 16; ++j) S[j] = 0ull;
@@ -1360,13 +1421,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     const StreamPos po = pos(co);
                     const int b = fdiv(po.bh, p.fd_H), h = po.bh - b * p.H;
                     const int t = walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row);
-                    if (t >= 0) {  // the row's columns inside Dv (padded columns stay behind)
-                        const int col0 = 64 * po.vb + ch0;
-                        uint4 *dst = reinterpret_cast<uint4 *>(out + (((size_t)b * p.T + t) * p.H + h) * p.Dv + col0);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (col0 + 8 * q < p.Dv) dst[q] = make_uint4(ow[4 * q], ow[4 * q + 1], ow[4 * q + 2], ow[4 * q + 3]);
-                    }
+                    store_row<E, NH == 1 || MODE == kFull>(p, ow, b, h, t, 64 * po.vb + ch0);
                 }
             }
             if (kBal && piece == 0 && b_chi > 0 && named_barrier_or(3, 128, !ok)) ok = false;
