@@ -210,15 +210,6 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// log sigma(x) = min(x, 0) - log(1 + e), e = e^{-|x|} in (0, 1]: log(1 + e) by the fast
-// logarithm (absolute error below 2^-21 on [1, 2]), or by its series e - e^2 / 2 where e < 1e-3
-// (error below e^3 / 3), so that the relative error stays below 4e-4 before the gate is
-// rounded to fp16.  NaN propagates; x = +inf gives 0, x = -inf gives -inf.
-__device__ __forceinline__ float log_sigmoid(float x) {
-    const float e = ex2(-fabsf(x) * kLog2e);
-    const float l1p = e < 1.0e-3f ? e * fmaf(-0.5f, e, 1.f) : __logf(1.f + e);
-    return fminf(x, 0.f) - l1p;
-}
 __device__ __forceinline__ float to_tf32(float x) {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -239,6 +230,25 @@ __device__ __forceinline__ f2 ex2_pair(f2 a) {
 __device__ __forceinline__ f2 ex2_neg_pair(f2 a) {
     const float2 x = unpack2(a);
     return pack2(ex2(-x.x), ex2(-x.y));
+}
+
+// log sigma(x) = min(x, 0) - log(1 + e), e = e^{-|x|} in (0, 1], of a pair: log(1 + e) by the hardware's
+// log2 (absolute error below 2^-21 on [1, 2]), or by its series e - e^2 / 2 where e < 1e-3 (error below
+// e^3 / 3), so that the relative error stays below 4e-4 before the gate is rounded to fp16.  NaN
+// propagates; x = +inf gives 0, x = -inf gives -inf.  (A degree-6 polynomial for log(1 + e) / e is more
+// exact and as fast, but moves the fp32 state by 2e-5.)
+__device__ __forceinline__ f2 log_sigmoid_pair(f2 x) {
+    const float2 v = unpack2(x);
+    const float2 e = make_float2(ex2(-fabsf(v.x) * kLog2e), ex2(-fabsf(v.y) * kLog2e));
+    const f2 ep = pack2(e.x, e.y), one = pack2(1.f, 1.f);
+    const float2 y = unpack2(add2(one, ep));
+    float l0, l1;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l0) : "f"(y.x));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l1) : "f"(y.y));
+    const float2 lg = unpack2(mul2(pack2(l0, l1), pack2(0.693147182464599609375f, 0.693147182464599609375f)));
+    const float2 se = unpack2(mul2(ep, fma2(pack2(-0.5f, -0.5f), ep, one)));
+    const f2 l1p = pack2(e.x < 1.0e-3f ? se.x : lg.x, e.y < 1.0e-3f ? se.y : lg.y);
+    return fma2(pack2(-1.f, -1.f), l1p, pack2(fminf(v.x, 0.f), fminf(v.y, 0.f)));
 }
 
 template <typename E> struct Elem;
@@ -819,42 +829,25 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         bool ok = true;
         if (warp == 1) {
             const uint32_t idesc_a = instr_desc(Elem<GE>::fmt, 64, 64, 0, 1);
-            const uint32_t idesc_z = instr_desc(Elem<E>::fmt, 64, 64, 0, 1);  // a K-major, W2 MN-major
             const uint64_t dL = kdesc(smem_u32(smem + kOffL));
 
-            // GP: Z runs one chunk ahead of A = L G, so that the two gen groups compute their
-            // chunks' gates concurrently: iteration c issues Z(c), then A(c - 1) once the gen group
-            // of c - 1 wrote its gates.  Z(c) reuses the A buffer of chunk c - 2 (PURDY(c - 2): its
-            // A was read), A(c - 1) overwrites Z(c - 1) (GRDY(c - 1): Z was read).
-            for (int c = 0; c < G + (GP ? 1 : 0); ++c) {
-                if (c < G) {
+            for (int c = 0; c < G; ++c) {
+                if constexpr (GP) {
+                    // the gen group wrote the chunk's gates (over its a tile, whose Z it has read)
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
+                    if (!ok) break;
+                } else {
                     if (c >= 2) {
                         ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], ((c - 2) >> 1) & 1, abort_flag, kWaitLimitNs));
                         if (!ok) break;
                     }
                     ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_FULL + c % kSlots], (c / kSlots) & 1, abort_flag, kWaitLimitNs));
                     if (!ok) break;
-                    tc_fence_after();
-                    if constexpr (GP) {
-                        // Z = a W2 (M = 64 tokens, N = 64 channels, K = r = 16: one MMA) into the
-                        // chunk's A buffer; a tile K-major with 128-byte rows, W2 MN-major
-                        const uint64_t da = kdesc(slot0 + (c % kSlots) * kSlotBytes + kG);
-                        const uint64_t dw = mndesc(smem_u32(smem + kOffW2) + (fdiv(c, p.fd_L) & 1) * kW2Bytes);
-                        mma_f16_ss_warp(tmem + kColA + (c & 1) * 64, da, dw, idesc_z, 0);
-                        mma_commit_warp(&bars[BAR_ZFULL + (c & 1)]);
-                    }
                 }
-                const int ca = GP ? c - 1 : c;  // the chunk whose A = L G goes now
-                if (ca < 0) continue;
-                if constexpr (GP) {
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (ca & 1)], (ca >> 1) & 1, abort_flag, kWaitLimitNs));
-                    if (!ok) break;
-                    tc_fence_after();
-                }
-                const uint64_t dg = mndesc(slot0 + (ca % kSlots) * kSlotBytes + kG);
-                const uint32_t d = tmem + kColA + (ca & 1) * 64;
-                mma4_f16_ss_warp<2, 128>(d, dL, dg, idesc_a, 0);
-                mma_commit_warp(&bars[BAR_AFULL + (ca & 1)]);
+                tc_fence_after();
+                const uint64_t dg = mndesc(slot0 + (c % kSlots) * kSlotBytes + kG);
+                mma4_f16_ss_warp<2, 128>(tmem + kColA + (c & 1) * 64, dL, dg, idesc_a, 0);
+                mma_commit_warp(&bars[BAR_AFULL + (c & 1)]);
             }
         } else if (warp == 14) {
             const uint32_t idesc_p16 = instr_desc(kFmtF16, 64, 64, 0, 0);
@@ -862,10 +855,35 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             const uint32_t idesc_u = instr_desc(kFmtF16, 64, 64, 1, 1);
             const uint64_t dqh0 = kdesc(smem_u32(smem + kOffOp)), dkh0 = kdesc(smem_u32(smem + kOffOp + kTile32));
             int su = 0;
-            for (int c = 0; c < G; ++c) {
+            // GP: Z(c) = a W2 (M = 64 tokens, N = 64 channels, K = r = 16: one MMA) into chunk c's TMEM A
+            // buffer; a tile K-major with 128-byte rows, W2 MN-major
+            auto issue_z = [&](int c) {
+                const uint64_t da = kdesc(slot0 + (c % kSlots) * kSlotBytes + kG);
+                const uint64_t dw = mndesc(smem_u32(smem + kOffW2) + (fdiv(c, p.fd_L) & 1) * kW2Bytes);
+                mma_f16_ss_warp(tmem + kColA + (c & 1) * 64, da, dw, instr_desc(Elem<E>::fmt, 64, 64, 0, 1), 0);
+                mma_commit_warp(&bars[BAR_ZFULL + (c & 1)]);
+            };
+            auto full = [&](int c) -> uint64_t * { return &bars[BAR_FULL + c % kSlots]; };
+            if constexpr (GP) {
+                for (int c = 0; c < 2 && c < G; ++c) {
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, kWaitLimitNs));
+                    if (!ok) break;
+                    tc_fence_after();
+                    issue_z(c);
+                }
+            }
+            for (int c = 0; ok && c < G; ++c) {
                 ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
                 if (!ok) break;
                 tc_fence_after();
+                // GP: chunk c + 2's Z reuses the A buffer that gen(c) has read.  It goes before P(c) and
+                // U(c) when the chunk has landed (the gen group forms those gates while it waits for P(c)),
+                // else after them.
+                bool z_due = GP && c + 2 < G;
+                if (z_due && !__any_sync(0xffffffffu, !mbar_test(full(c + 2), ((c + 2) / kSlots) & 1))) {
+                    issue_z(c + 2);
+                    z_due = false;
+                }
                 const uint32_t st = slot0 + su * kSlotBytes;
                 const uint32_t mode = __shfl_sync(0xffffffffu, mode_s[su], 0);
                 const uint32_t dp = tmem + kColP + (c & 1) * 64;
@@ -890,6 +908,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 mma4_f16_ss_warp<128, 128>(du, dk, dv, idesc_u, 0);
                 mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
                 su = (su == kSlots - 1) ? 0 : su + 1;
+                if (z_due) {
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(full(c + 2), ((c + 2) / kSlots) & 1, abort_flag, kWaitLimitNs));
+                    if (!ok) break;
+                    tc_fence_after();
+                    issue_z(c + 2);
+                }
             }
         } else if (!kSum) {
             const uint32_t idesc_o = instr_desc(kFmtF16, 64, 64, 0, 1);
@@ -982,48 +1006,53 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             store_row<E, true>(p, ow, b, h, t, 64 * po.vb + ch0);
             return true;
         };
+        // GP: chunk cz's gates from Z = a W2 (Sec. 3.1): g = logsigmoid(z + b) / tau in fp32, written as
+        // fp16 over the a tile, whose Z product has completed; rows outside the sequence keep g = 0 (no
+        // decay), as zero-filled gate rows do.  Done while the group waits for its previous chunk's
+        // scores, so that A = L G is ready when that chunk is finished (before, its round trip and the
+        // gates stood at the start of every chunk: GB300, B = 32, H = 12, 40 x 40 bf16 182 -> 127 us).
+        auto make_gates = [&](int cz) -> bool {
+            const int zb = cz & 1;
+            if (!mbar_wait(&bars[BAR_ZFULL + zb], (cz >> 1) & 1, abort_flag, kWaitLimitNs)) return false;
+            tc_fence_after();
+            uint8_t *gt = smem + kOffSlot + (cz % kSlots) * kSlotBytes + kG;
+            uint32_t zr[32];
+            tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + zb * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&zr[0]));
+            tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + zb * 64 + 16, *reinterpret_cast<uint32_t(*)[16]>(&zr[16]));
+            tmem_ld_wait();
+            const StreamPos pz = pos(cz);
+            const int wz = chunk_w0(p.order, p.T, pz.c) + row;
+            const uint32_t live = wz >= 0 && wz < p.T ? 0xffffffffu : 0u;
+            const float *bz = p.gbias + (size_t)(pz.bh - fdiv(pz.bh, p.fd_H) * p.H) * p.Dk;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                // 8 channels of the bias (Dk is a multiple of 8: all inside it or all past it)
+                float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
+                if (ch0 + 8 * q < p.Dk) {
+                    b0 = __ldg(reinterpret_cast<const float4 *>(bz + ch0 + 8 * q));
+                    b1 = __ldg(reinterpret_cast<const float4 *>(bz + ch0 + 8 * q + 4));
+                }
+                const f2 bq[4] = {pack2(b0.x, b0.y), pack2(b0.z, b0.w), pack2(b1.x, b1.y), pack2(b1.z, b1.w)};
+                uint32_t gq[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    gq[e] = h2bits(mul2(log_sigmoid_pair(add2(pack2(zr[8 * q + 2 * e], zr[8 * q + 2 * e + 1]), bq[e])),
+                                        pack2(p.tau_inv, p.tau_inv))) & live;
+                *reinterpret_cast<uint4 *>(gt + sw128(row, (ch0 + 8 * q) * 2)) = make_uint4(gq[0], gq[1], gq[2], gq[3]);
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars[BAR_GRDY + zb]);  // this warp's rows of G are in smem
+            return true;
+        };
+        bool zfail = false;
+        if constexpr (GP) zfail = gw < G && !make_gates(gw);
         int last_c = -1;  // the group's last chunk completed (its outputs are stored after the loop)
         for (int c = gw; c < G; c += 2) {
             const int sl = c % kSlots, bb = c & 1;
             const uint32_t ph = (c >> 1) & 1;
             uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
-            bool zfail = false;
-            if constexpr (GP) {
-                // the chunk's gates from Z = a W2 (Sec. 3.1): g = logsigmoid(z + b) / tau in fp32,
-                // written as fp16 over the a tile, whose Z product has completed; rows outside
-                // the sequence keep g = 0 (no decay), as zero-filled gate rows do
-                zfail = !mbar_wait(&bars[BAR_ZFULL + bb], ph, abort_flag, kWaitLimitNs);
-                tc_fence_after();
-                uint32_t zr[32];
-                tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + bb * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&zr[0]));
-                tmem_ld_16x32bx2_x16(tmem + lane_base + kColA + bb * 64 + 16, *reinterpret_cast<uint32_t(*)[16]>(&zr[16]));
-                tmem_ld_wait();
-                const StreamPos pz = pos(c);
-                const int wz = chunk_w0(p.order, p.T, pz.c) + row;
-                const bool live = wz >= 0 && wz < p.T;
-                const float *bz = p.gbias + (size_t)(pz.bh - fdiv(pz.bh, p.fd_H) * p.H) * p.Dk;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    // 8 channels of the bias (Dk is a multiple of 8: all inside it or all past it)
-                    float bq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    if (ch0 + 8 * q < p.Dk) {
-                        *reinterpret_cast<float4 *>(&bq[0]) = __ldg(reinterpret_cast<const float4 *>(bz + ch0 + 8 * q));
-                        *reinterpret_cast<float4 *>(&bq[4]) = __ldg(reinterpret_cast<const float4 *>(bz + ch0 + 8 * q + 4));
-                    }
-                    uint32_t gq[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float g0 = live ? log_sigmoid(__uint_as_float(zr[8 * q + 2 * e]) + bq[2 * e]) * p.tau_inv : 0.f;
-                        const float g1 = live ? log_sigmoid(__uint_as_float(zr[8 * q + 2 * e + 1]) + bq[2 * e + 1]) * p.tau_inv : 0.f;
-                        gq[e] = h2bits(g0, g1);
-                    }
-                    *reinterpret_cast<uint4 *>(st + kG + sw128(row, (ch0 + 8 * q) * 2)) = make_uint4(gq[0], gq[1], gq[2], gq[3]);
-                }
-                fence_proxy_async_smem();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bars[BAR_GRDY + bb]);  // this warp's rows of G are in smem
-            }
             const bool fail = zfail || !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
             // bf16 values become fp16 MMA operands in place (exact for |v| in the fp16
             // normal range); the loads go first so that their latency hides behind the
@@ -1169,6 +1198,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_PURDY + bb]);  // operands in smem, A(c) read
             if (kSum) continue;  // no scores
+            if constexpr (GP) zfail = c + 2 < G && !make_gates(c + 2);
             // ---- outputs of the group's previous chunk c-2 (O(c) reuses its TMEM buffer only
             // after ORDY(c), which this group signals below)
             bool ofail = false;
