@@ -39,6 +39,8 @@ def lib_path() -> str:
 def load(path: Optional[str] = None):
     """Load the CUDA library (built by ``__graft_entry__.build()``)."""
     global _lib
+    if path is None and _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -96,9 +98,17 @@ def load(path: Optional[str] = None):
         return lib
 
 
+# The current stream's handle without building a torch.cuda.Stream object, which took 3 us of a
+# 17 us host path (one 640^2 image's calls take 5 to 15 us on the GPU).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch._C._cuda_getDevice())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 def _dims(q, v, grid_h, grid_w):
@@ -108,6 +118,13 @@ def _dims(q, v, grid_h, grid_w):
     if T != grid_h * grid_w:
         raise ValueError(f"T={T} != grid_h*grid_w={grid_h * grid_w}")
     return B, H, Dk, v.shape[3]
+
+
+def _state(final_state, q, B, H, Dk, Dv):
+    """The final state's tensor: allocated (True), none, or the caller's."""
+    if final_state is True:
+        return torch.empty((B, H, Dk, Dv), dtype=torch.float32, device=q.device)
+    return final_state if isinstance(final_state, torch.Tensor) else None
 
 
 def _check(status: int, what: str, lib) -> None:
@@ -134,26 +151,26 @@ def forward(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, log_gate: torch.T
     preallocated [B, H, Dk, Dv] float32 tensor.  Returns (out, final_state).
     """
     lib = load()
-    for name, t in (("q", q), ("k", k), ("v", v), ("log_gate", log_gate)):
+    dtype = q.dtype
+    for t in (q, k, v, log_gate):
         if not t.is_cuda or not t.is_contiguous():
+            name = next(n for n, x in (("q", q), ("k", k), ("v", v), ("log_gate", log_gate)) if x is t)
             raise ValueError(f"{name} must be a contiguous CUDA tensor")
-        if t.dtype != q.dtype:
+        if t.dtype != dtype:
             raise ValueError("all inputs must share one dtype")
-    if q.dtype not in _DTYPES:
-        raise ValueError(f"unsupported dtype {q.dtype}")
+    code = _DTYPES.get(dtype)
+    if code is None:
+        raise ValueError(f"unsupported dtype {dtype}")
     B, H, Dk, Dv = _dims(q, v, grid_h, grid_w)
     if out is None:
-        out = torch.empty(v.shape, dtype=v.dtype, device=v.device)
-    fs = None
-    if final_state is True:
-        fs = torch.empty((B, H, Dk, Dv), dtype=torch.float32, device=q.device)
-    elif isinstance(final_state, torch.Tensor):
-        fs = final_state
+        out = torch.empty(v.shape, dtype=dtype, device=v.device)
+    fs = _state(final_state, q, B, H, Dk, Dv)
     status = lib.gtr_gla_fwd_sched(
         q.data_ptr(), k.data_ptr(), v.data_ptr(), log_gate.data_ptr(), B, H, grid_h, grid_w,
-        Dk, Dv, order, _DTYPES[q.dtype], out.data_ptr(), fs.data_ptr() if fs is not None else None,
+        Dk, Dv, order, code, out.data_ptr(), fs.data_ptr() if fs is not None else None,
         SCHEDULES[schedule], _stream_ptr(stream))
-    _check(status, "gtr_gla_fwd", lib)
+    if status:
+        _check(status, "gtr_gla_fwd", lib)
     return out, fs
 
 
@@ -189,28 +206,31 @@ def sswiglu_dwconv(gate: torch.Tensor, value: torch.Tensor, weight: torch.Tensor
     stride is shared (e.g. the two halves of one [B, T, 2F] tensor); weight:
     [F, 3, 3] float32, bias: [F] float32 or None (CUDA).  Returns out [B, T, F]."""
     lib = load()
-    if gate.dim() != 3 or gate.shape != value.shape or gate.dtype != value.dtype:
+    dtype, shape = gate.dtype, gate.shape
+    if len(shape) != 3 or shape != value.shape or dtype != value.dtype:
         raise ValueError("gate and value must be [B, T, F] tensors of one dtype")
-    if gate.dtype not in _DTYPES:
-        raise ValueError(f"unsupported dtype {gate.dtype}")
-    B, T, F = gate.shape
+    code = _DTYPES.get(dtype)
+    if code is None:
+        raise ValueError(f"unsupported dtype {dtype}")
+    B, T, F = shape
     if T != grid_h * grid_w:
         raise ValueError("T must equal grid_h * grid_w")
-    if gate.stride(2) != 1 or value.stride(2) != 1 or gate.stride(1) != value.stride(1) or \
-            gate.stride(0) != T * gate.stride(1) or value.stride(0) != T * value.stride(1):
+    sg, sv = gate.stride(), value.stride()
+    if sg[2] != 1 or sv[2] != 1 or sg[1] != sv[1] or sg[0] != T * sg[1] or sv[0] != T * sv[1]:
         raise ValueError("gate and value need contiguous channels and one shared token stride")
     if not gate.is_cuda or not value.is_cuda or not weight.is_cuda:
         raise ValueError("inputs must be CUDA tensors")
-    if weight.dtype != torch.float32 or not weight.is_contiguous() or tuple(weight.shape) != (F, 3, 3):
+    if weight.dtype != torch.float32 or not weight.is_contiguous() or weight.shape != (F, 3, 3):
         raise ValueError("weight must be a contiguous [F, 3, 3] float32 tensor")
-    if bias is not None and (bias.dtype != torch.float32 or not bias.is_contiguous() or tuple(bias.shape) != (F,)):
+    if bias is not None and (bias.dtype != torch.float32 or not bias.is_contiguous() or bias.shape != (F,)):
         raise ValueError("bias must be a contiguous [F] float32 tensor")
     if out is None:
-        out = torch.empty((B, T, F), dtype=gate.dtype, device=gate.device)
-    status = lib.gtr_sswiglu_dwconv(gate.data_ptr(), value.data_ptr(), gate.stride(1), weight.data_ptr(),
+        out = torch.empty((B, T, F), dtype=dtype, device=gate.device)
+    status = lib.gtr_sswiglu_dwconv(gate.data_ptr(), value.data_ptr(), sg[1], weight.data_ptr(),
                                     bias.data_ptr() if bias is not None else None, B, grid_h, grid_w, F,
-                                    _DTYPES[gate.dtype], out.data_ptr(), _stream_ptr(stream))
-    _check(status, "gtr_sswiglu_dwconv", lib)
+                                    code, out.data_ptr(), _stream_ptr(stream))
+    if status:
+        _check(status, "gtr_sswiglu_dwconv", lib)
     return out
 
 
