@@ -493,7 +493,8 @@ __device__ __forceinline__ void store_row(const TcParams &p, const uint32_t (&ow
 // Exact scores for one chunk (extreme or non-finite log-decays): serial prefix
 // of the clamped gates, P[rho][sigma] = sum_i q k 2^{a_r,i - a_j,i} (j <= r) by
 // CUDA cores, Qtil = q 2^{a}, Kbar = k 2^{a_last - a}, and the chunk decay.
-template <typename E, typename GT>
+// SUM (summary passes): no scores and no queries, the q and gate tiles stay as they are.
+template <typename E, typename GT, bool SUM>
 __device__ __noinline__ void exact_chunk(uint8_t *tq, uint8_t *tk, uint8_t *tgate, float *as,
                                          float *decay, int rev, int tg, int bar_id) {
     if (tg < kD) {
@@ -512,7 +513,7 @@ __device__ __noinline__ void exact_chunk(uint8_t *tq, uint8_t *tk, uint8_t *tgat
     const int rho = tg >> 1, half = tg & 1;
     const int r = rev ? kC - 1 - rho : rho;
     uint32_t packed[16];
-    for (int jj = 0; jj < 16; ++jj) {
+    for (int jj = 0; jj < (SUM ? 0 : 16); ++jj) {
         float pv[2];
         for (int u = 0; u < 2; ++u) {
             const int sig = half * 32 + 2 * jj + u;
@@ -532,15 +533,17 @@ __device__ __noinline__ void exact_chunk(uint8_t *tq, uint8_t *tk, uint8_t *tgat
     }
     const int rho_last = rev ? 0 : kC - 1;
     named_barrier_sync(bar_id, 128);  // every q/k/gate read of this chunk is done
-    for (int jj = 0; jj < 16; ++jj)
+    for (int jj = 0; jj < (SUM ? 0 : 16); ++jj)
         *reinterpret_cast<uint32_t *>(tgate + sw128(rho, (half * 32 + 2 * jj) * 2)) = packed[jj];
     for (int i = half * 32; i < half * 32 + 32; i += 2) {
         const uint32_t o16 = sw128(rho, i * 2);
-        const float2 q2 = Elem<E>::unpack(*reinterpret_cast<const uint32_t *>(tq + o16));
         const float2 k2 = Elem<E>::unpack(*reinterpret_cast<const uint32_t *>(tk + o16));
         const float a0 = as[rho * kD + i], a1 = as[rho * kD + i + 1];
         const float l0 = as[rho_last * kD + i], l1 = as[rho_last * kD + i + 1];
-        *reinterpret_cast<uint32_t *>(tq + o16) = h2bits(q2.x * ex2(a0), q2.y * ex2(a1));
+        if (!SUM) {
+            const float2 q2 = Elem<E>::unpack(*reinterpret_cast<const uint32_t *>(tq + o16));
+            *reinterpret_cast<uint32_t *>(tq + o16) = h2bits(q2.x * ex2(a0), q2.y * ex2(a1));
+        }
         *reinterpret_cast<uint32_t *>(tk + o16) = h2bits(k2.x * ex2(l0 - a0), k2.y * ex2(l1 - a1));
     }
 }
@@ -550,7 +553,8 @@ __device__ __noinline__ void exact_chunk(uint8_t *tq, uint8_t *tk, uint8_t *tgat
 // Kbar = K^ c2 over k.  Re-reads the thread's 32 log-decays from TMEM (A is kept
 // until the operands are built): out of line, this rarer path leaves the fp16 path's
 // code and registers as they are (inlined it cost workload 2 6 %).
-template <typename E>
+// SUM (summary passes): only Kbar.
+template <typename E, bool SUM>
 __device__ __noinline__ void tf32_operands(uint8_t *tq, uint8_t *tk, uint8_t *opbuf, const float *ref,
                                            uint32_t taddr, int row, int ch0) {
     uint32_t ar[32];
@@ -562,7 +566,7 @@ __device__ __noinline__ void tf32_operands(uint8_t *tq, uint8_t *tk, uint8_t *op
     for (int g8 = 0; g8 < 4; ++g8) {
         const int cl = ch0 + 8 * g8;
         const uint32_t o16 = sw128(row, cl * 2);
-        const uint4 qw = *reinterpret_cast<const uint4 *>(tq + o16);
+        const uint4 qw = SUM ? make_uint4(0u, 0u, 0u, 0u) : *reinterpret_cast<const uint4 *>(tq + o16);
         const uint4 kw = *reinterpret_cast<const uint4 *>(tk + o16);
         const uint32_t qa[4] = {qw.x, qw.y, qw.z, qw.w}, ka[4] = {kw.x, kw.y, kw.z, kw.w};
         // A_mid log2, c1 and c2 of the 8 channels (16-byte aligned rows of the references)
@@ -586,21 +590,23 @@ __device__ __noinline__ void tf32_operands(uint8_t *tq, uint8_t *tk, uint8_t *op
             ks[2 * e] = k2.x * ex2(-e0);
             ks[2 * e + 1] = k2.y * ex2(-e1);
         }
-        *reinterpret_cast<float4 *>(qh + off32(row, cl)) =
-            make_float4(to_tf32(qs[0]), to_tf32(qs[1]), to_tf32(qs[2]), to_tf32(qs[3]));
-        *reinterpret_cast<float4 *>(qh + off32(row, cl + 4)) =
-            make_float4(to_tf32(qs[4]), to_tf32(qs[5]), to_tf32(qs[6]), to_tf32(qs[7]));
-        *reinterpret_cast<float4 *>(kh + off32(row, cl)) =
-            make_float4(to_tf32(ks[0]), to_tf32(ks[1]), to_tf32(ks[2]), to_tf32(ks[3]));
-        *reinterpret_cast<float4 *>(kh + off32(row, cl + 4)) =
-            make_float4(to_tf32(ks[4]), to_tf32(ks[5]), to_tf32(ks[6]), to_tf32(ks[7]));
+        if (!SUM) {
+            *reinterpret_cast<float4 *>(qh + off32(row, cl)) =
+                make_float4(to_tf32(qs[0]), to_tf32(qs[1]), to_tf32(qs[2]), to_tf32(qs[3]));
+            *reinterpret_cast<float4 *>(qh + off32(row, cl + 4)) =
+                make_float4(to_tf32(qs[4]), to_tf32(qs[5]), to_tf32(qs[6]), to_tf32(qs[7]));
+            *reinterpret_cast<float4 *>(kh + off32(row, cl)) =
+                make_float4(to_tf32(ks[0]), to_tf32(ks[1]), to_tf32(ks[2]), to_tf32(ks[3]));
+            *reinterpret_cast<float4 *>(kh + off32(row, cl + 4)) =
+                make_float4(to_tf32(ks[4]), to_tf32(ks[5]), to_tf32(ks[6]), to_tf32(ks[7]));
+        }
         uint32_t qo[4], ko[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             qo[e] = h2bits(qs[2 * e] * c1v[2 * e], qs[2 * e + 1] * c1v[2 * e + 1]);
             ko[e] = h2bits(ks[2 * e] * c2v[2 * e], ks[2 * e + 1] * c2v[2 * e + 1]);
         }
-        *reinterpret_cast<uint4 *>(tq + o16) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
+        if (!SUM) *reinterpret_cast<uint4 *>(tq + o16) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
         *reinterpret_cast<uint4 *>(tk + o16) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
     }
 }
@@ -652,8 +658,14 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     constexpr bool kRollBuild = !kGenOut;
     const int N = p.n_chunks;   // chunks per sequence
     const int L = p.seg_len;    // chunks per unit
-    constexpr int nh = NH;   // 64-channel key halves per chunk (Dk / 64)
-    constexpr int lognv = NV - 1;  // 64-column value slices per sequence (Dv / 64): 1 or 2
+    // Summaries of two key halves: a unit is one half with every value slice (else one value slice
+    // with every key half), so that a chunk's A and Kbar are built once instead of once per slice.  The
+    // second slice of v takes the q tile's place, its U the O columns (neither is used by a summary),
+    // its state the other half's registers.  GB300, Dk = Dv = 128, 128 x 128, B = 2, H = 8: 252 -> 219 us both passes.
+    constexpr bool kHalfSum = kSum && NH == 2;
+    constexpr int kSlices = kHalfSum ? NV : 1;  // value slices per virtual chunk
+    constexpr int nh = kHalfSum ? 1 : NH;   // 64-channel key halves per chunk (Dk / 64) of a unit
+    constexpr int lognv = kHalfSum ? 1 : NV - 1;  // units per (sequence, segment): 64-column value slices, or key halves
     constexpr int kDk = 64 * NH, kDv = 64 * NV;
     // this CTA's stream of virtual chunks: every barrier phase, stage slot and TMEM
     // buffer below follows the stream index (O: the real chunk's index), so
@@ -667,7 +679,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                               static_cast<int>(gridDim.x));
     auto pos = [&](int v) -> StreamPos {
         if constexpr (kBal) return stream_pos_bal(v, N, lognv, b_head, b_full, b_tail, b_chi, b_t0, p.bal_n);
-        else return stream_pos(v, L, nh, lognv, p.fd_per, kSplit, p.fd_nsu);
+        StreamPos ps = stream_pos(v, L, nh, lognv, p.fd_per, kSplit, p.fd_nsu);
+        if constexpr (kHalfSum) {
+            ps.a = ps.vb;
+            ps.vb = 0;
+        }
+        return ps;
     };
     const int rev = p.order & 1;
 
@@ -781,7 +798,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     // buffer of the unit's parity (the unit before last, whose Z products used it,
                     // ended at least four chunks earlier: its last Z completed before this slot freed)
                     const bool w2 = GP && ps.cl == 0;
-                    mbar_arrive_expect_tx(fb, (kSum ? kSlotBytes - kTile16 : kSlotBytes) + (w2 ? kW2Bytes : 0));
+                    mbar_arrive_expect_tx(fb, (kSum && kSlices == 1 ? kSlotBytes - kTile16 : kSlotBytes) + (w2 ? kW2Bytes : 0));
                     if (w2) tma_load_5d(smem + kOffW2 + (fdiv(g, p.fd_L) & 1) * kW2Bytes, &p.w2map, fb, 0, 0, h, 0, 0);
                     int x0, y0;
                     if (chunk_walk_start(p.order, p.T, p.fd_gh, c, &x0, &y0)) {
@@ -791,11 +808,13 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         if (!kSum) tma_load_im2col_5d(st + kQ, &p.cmaps[T_Q], fb, xk, y0, x0, h, b);
                         tma_load_im2col_5d(st + kK, &p.cmaps[T_K], fb, xk, y0, x0, h, b);
                         tma_load_im2col_5d(st + kV, &p.cmaps[T_V], fb, xv, y0, x0, h, b);
+                        if (kSlices == 2) tma_load_im2col_5d(st + kQ, &p.cmaps[T_V], fb, 64, y0, x0, h, b);
                         tma_load_im2col_5d(st + kG, &p.cmaps[T_G], fb, GP ? 0 : xk, y0, x0, GP ? 0 : h, b);
                     } else chunk_load_boxes(p.order, p.T, p.fd_gh, p.grid_w, c, [&](int hi, int row, int c2, int c3) {
                         if (!kSum) tma_load_5d(st + kQ + row * 128, &p.maps[T_Q][hi], fb, xk, h, c2, c3, b);
                         tma_load_5d(st + kK + row * 128, &p.maps[T_K][hi], fb, xk, h, c2, c3, b);
                         tma_load_5d(st + kV + row * 128, &p.maps[T_V][hi], fb, xv, h, c2, c3, b);
+                        if (kSlices == 2) tma_load_5d(st + kQ + row * 128, &p.maps[T_V][hi], fb, 64, h, c2, c3, b);
                         // the gate tile, or (gate producer) the 16 projection values of each token,
                         // zero-filled to a 128-byte row
                         tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], fb, GP ? 0 : xk, GP ? 0 : h, c2, c3, b);
@@ -906,6 +925,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint64_t dk = mndesc(st + kK), dv = mndesc(st + kV);
                 const uint32_t du = tmem + kColU + (c & 1) * 64;
                 mma4_f16_ss_warp<128, 128>(du, dk, dv, idesc_u, 0);
+                if (kSlices == 2) mma4_f16_ss_warp<128, 128>(tmem + kColO + (c & 1) * 64, dk, mndesc(st + kQ), idesc_u, 0);
                 mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
                 su = (su == kSlots - 1) ? 0 : su + 1;
                 if (z_due) {
@@ -1164,24 +1184,28 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 }
             } else if (!opfail) {
                 if (mode == kModeTF32)
-                    tf32_operands<E>(tq, tk, smem + kOffOp + gw * 2 * kTile32, ref, ta, row, ch0);
+                    tf32_operands<E, kSum>(tq, tk, smem + kOffOp + gw * 2 * kTile32, ref, ta, row, ch0);
                 else
-                    exact_chunk<E, GE>(tq, tk, tgt, reinterpret_cast<float *>(smem + kOffOp + gw * 2 * kTile32), decay_s + sl * kD, rev, tg,
+                    exact_chunk<E, GE, kSum>(tq, tk, tgt, reinterpret_cast<float *>(smem + kOffOp + gw * 2 * kTile32), decay_s + sl * kD, rev, tg,
                                    bar_id);
             }
             if constexpr (std::is_same<E, __nv_bfloat16>::value) {
-                uint4 vw[4];
+#pragma unroll 1
+                for (int vs = 0; vs < kSlices; ++vs) {
+                    uint8_t *tv = vs == 0 ? st + kV : st + kQ;
+                    uint4 vw[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) vw[q] = *reinterpret_cast<const uint4 *>(st + kV + sw128(row, (ch0 + 8 * q) * 2));
+                    for (int q = 0; q < 4; ++q) vw[q] = *reinterpret_cast<const uint4 *>(tv + sw128(row, (ch0 + 8 * q) * 2));
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t *wp = reinterpret_cast<uint32_t *>(&vw[q]);
+                    for (int q = 0; q < 4; ++q) {
+                        uint32_t *wp = reinterpret_cast<uint32_t *>(&vw[q]);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 fv = Elem<E>::unpack(wp[e]);
-                        wp[e] = h2bits(fv.x, fv.y);
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 fv = Elem<E>::unpack(wp[e]);
+                            wp[e] = h2bits(fv.x, fv.y);
+                        }
+                        *reinterpret_cast<uint4 *>(tv + sw128(row, (ch0 + 8 * q) * 2)) = vw[q];
                     }
-                    *reinterpret_cast<uint4 *>(st + kV + sw128(row, (ch0 + 8 * q) * 2)) = vw[q];
                 }
             }
             fence_proxy_async_smem();
@@ -1383,6 +1407,13 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
 #pragma unroll
                         for (int hf = 0; hf < 2; ++hf) {
                             uint32_t r[16];
+                            if constexpr (kSlices == 2) {
+                                tmem_ld_16x32bx2_x16(tmem + lane_base + kColO + bb * 64 + 16 * hf, r);
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    So[8 * hf + j] = fma2(pack2(dc, dc), So[8 * hf + j], mul2(pack2(c2, c2), pack2(r[2 * j], r[2 * j + 1])));
+                            }
                             tmem_ld_16x32bx2_x16(tmem + lane_base + kColU + bb * 64 + 16 * hf, r);
                             tmem_ld_wait();
 #pragma unroll
@@ -1405,6 +1436,10 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                             ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(base + (size_t)(64 * ps.a + row) * kDv + 64 * ps.vb + ch0);
 #pragma unroll
                             for (int j = 0; j < 8; ++j) dst[j] = make_ulonglong2(S[2 * j], S[2 * j + 1]);
+                            if constexpr (kSlices == 2) {
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) dst[16 + j] = make_ulonglong2(So[2 * j], So[2 * j + 1]);
+                            }
                             if (ps.vb == 0 && hc == 0) base[(size_t)kDk * kDv + 64 * ps.a + row] = dp;
                         }
                     } else if (ps.c == N - 1 && p.final_state != nullptr && 64 * ps.a + row < p.Dk) {
@@ -1417,7 +1452,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bars[BAR_PURDY + bb]);  // U(c) drained: counts for chunk c + 2
-                    if constexpr (NH == 2) {  // the other key half comes next
+                    if constexpr (NH == 2 && !kHalfSum) {  // the other key half comes next
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const f2 t = S[j];
@@ -1899,7 +1934,6 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.nseg = nseg;
     tp.seg_len = sp.len;
     tp.fd_L = make_fastdiv(sp.len);
-    tp.fd_per = make_fastdiv(sp.len * tp.nh);
     tp.summary = static_cast<float *>(workspace);
     tp.flags = nullptr;
     tp.epoch = 0;
@@ -1911,9 +1945,11 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     // persistent: one CTA per SM, each walking its share of the work units
     unsigned sum_ctas = 0;
     if (nseg > 1) {  // pass 1: end state from zero and total decay of segments 0 .. nseg-2
+        // (two key halves: a unit is one half with every value slice)
         tp.nsu = nseg - 1;
         tp.fd_nsu = make_fastdiv(tp.nsu);
-        tp.n_units = seqs * tp.nsu;
+        tp.n_units = (tp.nh == 2 ? 2 * static_cast<int>(p.B * p.H) : seqs) * tp.nsu;
+        tp.fd_per = make_fastdiv(sp.len);
         const dim3 grid(static_cast<unsigned>(tp.n_units < n_sm ? tp.n_units : n_sm));
         sum_ctas = grid.x;
         e = half ? launch_shape<__half, kSummary>(grid, tp, stream) : launch_shape<__nv_bfloat16, kSummary>(grid, tp, stream);
@@ -1923,6 +1959,7 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.nsu = nseg;
     tp.fd_nsu = make_fastdiv(nseg);
     tp.n_units = seqs * nseg;
+    tp.fd_per = make_fastdiv(sp.len * tp.nh);
     if (nseg == 1 && bal && workspace != nullptr && workspace_bytes >= handoff_bytes(n_sm)) {
         // equal contiguous chunk ranges, one CTA per SM
         r.ran = kRanTcBalanced;
