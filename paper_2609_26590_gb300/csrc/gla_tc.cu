@@ -51,6 +51,7 @@
 //                (GENOUT launches: the gen warpgroup that built the chunk stores them).
 //   warp 14      issuer of P(c) and U(c).
 //   warp 15      issuer of O(c).
+// (Two key halves: warps 0-3 producer, A, P/U and O issuers, 4-7 and 8-11 gen, 12-15 epi.)
 // Each issuer waits only for the inputs of its own product, so the issue overhead
 // of one product does not hold up the others.
 // A warp reads the TMEM lanes of sub-partition (warp % 4); an M = 64 accumulator
@@ -630,6 +631,15 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     volatile uint32_t *mode_s = reinterpret_cast<volatile uint32_t *>(smem + kOffMode);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // Two key halves: the epi holds two states and spills at the 128 registers a thread of 512 gets, so
+    // the roles are aligned to warpgroups (0-3 producer and issuers, 4-11 gen, 12-15 epi) and the
+    // control warps' registers go to the others (GB300, Dk = Dv = 128: 128 x 128 images 219 -> 202 us,
+    // B = 16, H = 12, 40 x 40 185 -> 163 us).  With one key half nothing spills, and the roles as listed
+    // at the top measured faster (6,400 tokens, tf32 scores: 159 us against 164 aligned).
+    constexpr bool kAligned = NH == 2;
+    constexpr int kGen0 = kAligned ? 4 : 2, kEpi0 = kAligned ? 12 : 10, kWarpPU = kAligned ? 2 : 14;
+    constexpr uint32_t kRegsCtl = 64, kRegsGen = 136, kRegsEpi = 176;
+    static_assert(kRegsCtl + 2 * kRegsGen + kRegsEpi == 4 * 128, "the registers of the launch");
     // the output pass after a summary pass may start now: its CTAs set up (barriers, TMEM) on
     // the free SMs and wait for this grid only before they read the summaries
     if constexpr (MODE == kSummary) pdl_launch_dependents();
@@ -712,9 +722,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         tmem_alloc(const_cast<uint32_t *>(tmem_base_s), kTmemCols);
         tmem_relinquish();
     }
-    if (warp >= 2 && warp < 6) {
+    if (warp >= kGen0 && warp < kGen0 + 4) {
         // triangle of ones in scan order: L[rho][sigma] = 1 when sigma is at or before rho
-        const int tg = threadIdx.x - 64;
+        const int tg = threadIdx.x - 32 * kGen0;
         const int rho = tg >> 1, half = tg & 1;
         uint8_t *L = smem + kOffL;
 #pragma unroll
@@ -778,190 +788,194 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     tc_fence_after();
     const uint32_t tmem = *tmem_base_s;
 
-    if (warp == 0) {
-        // ======================================================= TMA producer
-        if (lane == 0) {
-            int issued = 0;
-            for (int g = 0; g < G; ++g) {
-                const int sl = g % kSlots;
-                const StreamPos ps = pos(g);
-                const int b = fdiv(ps.bh, p.fd_H), h = ps.bh - b * p.H, c = ps.c;
-                const int xk = 64 * ps.a, xv = 64 * ps.vb;  // channel offsets of the key half, value slice
-                if (!mbar_wait(&bars[BAR_EMPTY + sl], ((g / kSlots) & 1) ^ 1, abort_flag, kWaitLimitNs)) {
-                    record_timeout(abort_flag);
-                    break;
+    if (kAligned ? warp < 4 : (warp < 2 || warp >= 14)) {
+        if constexpr (kAligned) setmaxnreg_dec<kRegsCtl>();
+        if (warp == 0) {
+            // ======================================================= TMA producer
+            if (lane == 0) {
+                int issued = 0;
+                for (int g = 0; g < G; ++g) {
+                    const int sl = g % kSlots;
+                    const StreamPos ps = pos(g);
+                    const int b = fdiv(ps.bh, p.fd_H), h = ps.bh - b * p.H, c = ps.c;
+                    const int xk = 64 * ps.a, xv = 64 * ps.vb;  // channel offsets of the key half, value slice
+                    if (!mbar_wait(&bars[BAR_EMPTY + sl], ((g / kSlots) & 1) ^ 1, abort_flag, kWaitLimitNs)) {
+                        record_timeout(abort_flag);
+                        break;
+                    }
+                    uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
+                    uint64_t *fb = &bars[BAR_FULL + sl];
+                    if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
+                        // gate producer: a unit's first chunk also brings the head's W2 block, into the
+                        // buffer of the unit's parity (the unit before last, whose Z products used it,
+                        // ended at least four chunks earlier: its last Z completed before this slot freed)
+                        const bool w2 = GP && ps.cl == 0;
+                        mbar_arrive_expect_tx(fb, (kSum && kSlices == 1 ? kSlotBytes - kTile16 : kSlotBytes) + (w2 ? kW2Bytes : 0));
+                        if (w2) tma_load_5d(smem + kOffW2 + (fdiv(g, p.fd_L) & 1) * kW2Bytes, &p.w2map, fb, 0, 0, h, 0, 0);
+                        int x0, y0;
+                        if (chunk_walk_start(p.order, p.T, p.fd_gh, c, &x0, &y0)) {
+                            // column orders, chunk inside the sequence: one im2col walk per tensor
+                            // (boxes per column segment cost the TMA unit one request each and ran
+                            // up to 1.9x slower)
+                            if (!kSum) tma_load_im2col_5d(st + kQ, &p.cmaps[T_Q], fb, xk, y0, x0, h, b);
+                            tma_load_im2col_5d(st + kK, &p.cmaps[T_K], fb, xk, y0, x0, h, b);
+                            tma_load_im2col_5d(st + kV, &p.cmaps[T_V], fb, xv, y0, x0, h, b);
+                            if (kSlices == 2) tma_load_im2col_5d(st + kQ, &p.cmaps[T_V], fb, 64, y0, x0, h, b);
+                            tma_load_im2col_5d(st + kG, &p.cmaps[T_G], fb, GP ? 0 : xk, y0, x0, GP ? 0 : h, b);
+                        } else chunk_load_boxes(p.order, p.T, p.fd_gh, p.grid_w, c, [&](int hi, int row, int c2, int c3) {
+                            if (!kSum) tma_load_5d(st + kQ + row * 128, &p.maps[T_Q][hi], fb, xk, h, c2, c3, b);
+                            tma_load_5d(st + kK + row * 128, &p.maps[T_K][hi], fb, xk, h, c2, c3, b);
+                            tma_load_5d(st + kV + row * 128, &p.maps[T_V][hi], fb, xv, h, c2, c3, b);
+                            if (kSlices == 2) tma_load_5d(st + kQ + row * 128, &p.maps[T_V][hi], fb, 64, h, c2, c3, b);
+                            // the gate tile, or (gate producer) the 16 projection values of each token,
+                            // zero-filled to a 128-byte row
+                            tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], fb, GP ? 0 : xk, GP ? 0 : h, c2, c3, b);
+                        });
+                    }
+                    ++issued;
                 }
-                uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
-                uint64_t *fb = &bars[BAR_FULL + sl];
-                if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
-                    // gate producer: a unit's first chunk also brings the head's W2 block, into the
-                    // buffer of the unit's parity (the unit before last, whose Z products used it,
-                    // ended at least four chunks earlier: its last Z completed before this slot freed)
-                    const bool w2 = GP && ps.cl == 0;
-                    mbar_arrive_expect_tx(fb, (kSum && kSlices == 1 ? kSlotBytes - kTile16 : kSlotBytes) + (w2 ? kW2Bytes : 0));
-                    if (w2) tma_load_5d(smem + kOffW2 + (fdiv(g, p.fd_L) & 1) * kW2Bytes, &p.w2map, fb, 0, 0, h, 0, 0);
-                    int x0, y0;
-                    if (chunk_walk_start(p.order, p.T, p.fd_gh, c, &x0, &y0)) {
-                        // column orders, chunk inside the sequence: one im2col walk per tensor
-                        // (boxes per column segment cost the TMA unit one request each and ran
-                        // up to 1.9x slower)
-                        if (!kSum) tma_load_im2col_5d(st + kQ, &p.cmaps[T_Q], fb, xk, y0, x0, h, b);
-                        tma_load_im2col_5d(st + kK, &p.cmaps[T_K], fb, xk, y0, x0, h, b);
-                        tma_load_im2col_5d(st + kV, &p.cmaps[T_V], fb, xv, y0, x0, h, b);
-                        if (kSlices == 2) tma_load_im2col_5d(st + kQ, &p.cmaps[T_V], fb, 64, y0, x0, h, b);
-                        tma_load_im2col_5d(st + kG, &p.cmaps[T_G], fb, GP ? 0 : xk, y0, x0, GP ? 0 : h, b);
-                    } else chunk_load_boxes(p.order, p.T, p.fd_gh, p.grid_w, c, [&](int hi, int row, int c2, int c3) {
-                        if (!kSum) tma_load_5d(st + kQ + row * 128, &p.maps[T_Q][hi], fb, xk, h, c2, c3, b);
-                        tma_load_5d(st + kK + row * 128, &p.maps[T_K][hi], fb, xk, h, c2, c3, b);
-                        tma_load_5d(st + kV + row * 128, &p.maps[T_V][hi], fb, xv, h, c2, c3, b);
-                        if (kSlices == 2) tma_load_5d(st + kQ + row * 128, &p.maps[T_V][hi], fb, 64, h, c2, c3, b);
-                        // the gate tile, or (gate producer) the 16 projection values of each token,
-                        // zero-filled to a 128-byte row
-                        tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], fb, GP ? 0 : xk, GP ? 0 : h, c2, c3, b);
-                    });
+                if (*abort_flag) {  // never leave while copies are still landing in shared memory
+                    for (int g = (issued > kSlots ? issued - kSlots : 0); g < issued; ++g)
+                        if (!(p.drop_load && blockIdx.x == 0 && g == 0))
+                            mbar_wait(&bars[BAR_FULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
                 }
-                ++issued;
             }
-            if (*abort_flag) {  // never leave while copies are still landing in shared memory
-                for (int g = (issued > kSlots ? issued - kSlots : 0); g < issued; ++g)
-                    if (!(p.drop_load && blockIdx.x == 0 && g == 0))
-                        mbar_wait(&bars[BAR_FULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
-            }
-        }
-    } else if (warp == 1 || warp >= 14) {
-        // ======================================================= MMA issuers
-        // Three warps issue the products, each in program order and waiting only for
-        // its own inputs, so that the issue overhead of one product never delays
-        // another.  A whole warp runs each loop (operands warp-uniform) and one
-        // elected lane issues each MMA.
-        //   warp 1   A(c) = L G          once chunk c landed and gen(c-2) built its
-        //                                operands (so TMEM A of the parity was read)
-        //   warp 14  P(c) = Q^ K^^T,     once PURDY(c): gen(c) operands in smem and epi
-        //            U(c) = Kbar^T V     drained U(c-2)
-        //   warp 15  O(c) = Q S'_[c] + P V   once ORDY(c)
-        // A tcgen05.commit tracks only its own thread's MMAs: the slot of chunk c is
-        // released by two commits, after U(c) (warp 14) and after O(c) (warp 15); P(c)
-        // and A(c) completed before ORDY(c).  No waiter can be overtaken by two phases
-        // of its barrier: PURDY(c + 2) needs A(c + 2) and U(c), FULL of the next chunk
-        // of a slot needs that slot's EMPTY, ORDY(c + 2) needs O(c) read.
-        const uint32_t slot0 = smem_u32(smem + kOffSlot);
-        bool ok = true;
-        if (warp == 1) {
-            const uint32_t idesc_a = instr_desc(Elem<GE>::fmt, 64, 64, 0, 1);
-            const uint64_t dL = kdesc(smem_u32(smem + kOffL));
+        } else {
+            // ======================================================= MMA issuers
+            // Three warps issue the products, each in program order and waiting only for
+            // its own inputs, so that the issue overhead of one product never delays
+            // another.  A whole warp runs each loop (operands warp-uniform) and one
+            // elected lane issues each MMA.
+            //   warp 1   A(c) = L G          once chunk c landed and gen(c-2) built its
+            //                                operands (so TMEM A of the parity was read)
+            //   warp 14  P(c) = Q^ K^^T,     once PURDY(c): gen(c) operands in smem and epi
+            //            U(c) = Kbar^T V     drained U(c-2)
+            //   warp 15  O(c) = Q S'_[c] + P V   once ORDY(c)
+            // A tcgen05.commit tracks only its own thread's MMAs: the slot of chunk c is
+            // released by two commits, after U(c) (warp 14) and after O(c) (warp 15); P(c)
+            // and A(c) completed before ORDY(c).  No waiter can be overtaken by two phases
+            // of its barrier: PURDY(c + 2) needs A(c + 2) and U(c), FULL of the next chunk
+            // of a slot needs that slot's EMPTY, ORDY(c + 2) needs O(c) read.
+            const uint32_t slot0 = smem_u32(smem + kOffSlot);
+            bool ok = true;
+            if (warp == 1) {
+                const uint32_t idesc_a = instr_desc(Elem<GE>::fmt, 64, 64, 0, 1);
+                const uint64_t dL = kdesc(smem_u32(smem + kOffL));
 
-            for (int c = 0; c < G; ++c) {
-                if constexpr (GP) {
-                    // the gen group wrote the chunk's gates (over its a tile, whose Z it has read)
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
-                    if (!ok) break;
-                } else {
-                    if (c >= 2) {
-                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], ((c - 2) >> 1) & 1, abort_flag, kWaitLimitNs));
+                for (int c = 0; c < G; ++c) {
+                    if constexpr (GP) {
+                        // the gen group wrote the chunk's gates (over its a tile, whose Z it has read)
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
+                        if (!ok) break;
+                    } else {
+                        if (c >= 2) {
+                            ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], ((c - 2) >> 1) & 1, abort_flag, kWaitLimitNs));
+                            if (!ok) break;
+                        }
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_FULL + c % kSlots], (c / kSlots) & 1, abort_flag, kWaitLimitNs));
                         if (!ok) break;
                     }
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_FULL + c % kSlots], (c / kSlots) & 1, abort_flag, kWaitLimitNs));
-                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dg = mndesc(slot0 + (c % kSlots) * kSlotBytes + kG);
+                    mma4_f16_ss_warp<2, 128>(tmem + kColA + (c & 1) * 64, dL, dg, idesc_a, 0);
+                    mma_commit_warp(&bars[BAR_AFULL + (c & 1)]);
                 }
-                tc_fence_after();
-                const uint64_t dg = mndesc(slot0 + (c % kSlots) * kSlotBytes + kG);
-                mma4_f16_ss_warp<2, 128>(tmem + kColA + (c & 1) * 64, dL, dg, idesc_a, 0);
-                mma_commit_warp(&bars[BAR_AFULL + (c & 1)]);
-            }
-        } else if (warp == 14) {
-            const uint32_t idesc_p16 = instr_desc(kFmtF16, 64, 64, 0, 0);
-            const uint32_t idesc_p32 = instr_desc(kFmtTF32, 64, 64, 0, 0);
-            const uint32_t idesc_u = instr_desc(kFmtF16, 64, 64, 1, 1);
-            const uint64_t dqh0 = kdesc(smem_u32(smem + kOffOp)), dkh0 = kdesc(smem_u32(smem + kOffOp + kTile32));
-            int su = 0;
-            // GP: Z(c) = a W2 (M = 64 tokens, N = 64 channels, K = r = 16: one MMA) into chunk c's TMEM A
-            // buffer; a tile K-major with 128-byte rows, W2 MN-major
-            auto issue_z = [&](int c) {
-                const uint64_t da = kdesc(slot0 + (c % kSlots) * kSlotBytes + kG);
-                const uint64_t dw = mndesc(smem_u32(smem + kOffW2) + (fdiv(c, p.fd_L) & 1) * kW2Bytes);
-                mma_f16_ss_warp(tmem + kColA + (c & 1) * 64, da, dw, instr_desc(Elem<E>::fmt, 64, 64, 0, 1), 0);
-                mma_commit_warp(&bars[BAR_ZFULL + (c & 1)]);
-            };
-            auto full = [&](int c) -> uint64_t * { return &bars[BAR_FULL + c % kSlots]; };
-            if constexpr (GP) {
-                for (int c = 0; c < 2 && c < G; ++c) {
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, kWaitLimitNs));
+            } else if (warp == kWarpPU) {
+                const uint32_t idesc_p16 = instr_desc(kFmtF16, 64, 64, 0, 0);
+                const uint32_t idesc_p32 = instr_desc(kFmtTF32, 64, 64, 0, 0);
+                const uint32_t idesc_u = instr_desc(kFmtF16, 64, 64, 1, 1);
+                const uint64_t dqh0 = kdesc(smem_u32(smem + kOffOp)), dkh0 = kdesc(smem_u32(smem + kOffOp + kTile32));
+                int su = 0;
+                // GP: Z(c) = a W2 (M = 64 tokens, N = 64 channels, K = r = 16: one MMA) into chunk c's TMEM A
+                // buffer; a tile K-major with 128-byte rows, W2 MN-major
+                auto issue_z = [&](int c) {
+                    const uint64_t da = kdesc(slot0 + (c % kSlots) * kSlotBytes + kG);
+                    const uint64_t dw = mndesc(smem_u32(smem + kOffW2) + (fdiv(c, p.fd_L) & 1) * kW2Bytes);
+                    mma_f16_ss_warp(tmem + kColA + (c & 1) * 64, da, dw, instr_desc(Elem<E>::fmt, 64, 64, 0, 1), 0);
+                    mma_commit_warp(&bars[BAR_ZFULL + (c & 1)]);
+                };
+                auto full = [&](int c) -> uint64_t * { return &bars[BAR_FULL + c % kSlots]; };
+                if constexpr (GP) {
+                    for (int c = 0; c < 2 && c < G; ++c) {
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, kWaitLimitNs));
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_z(c);
+                    }
+                }
+                for (int c = 0; ok && c < G; ++c) {
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
                     if (!ok) break;
                     tc_fence_after();
-                    issue_z(c);
+                    // GP: chunk c + 2's Z reuses the A buffer that gen(c) has read.  It goes before P(c) and
+                    // U(c) when the chunk has landed (the gen group forms those gates while it waits for P(c)),
+                    // else after them.
+                    bool z_due = GP && c + 2 < G;
+                    if (z_due && !__any_sync(0xffffffffu, !mbar_test(full(c + 2), ((c + 2) / kSlots) & 1))) {
+                        issue_z(c + 2);
+                        z_due = false;
+                    }
+                    const uint32_t st = slot0 + su * kSlotBytes;
+                    const uint32_t mode = __shfl_sync(0xffffffffu, mode_s[su], 0);
+                    const uint32_t dp = tmem + kColP + (c & 1) * 64;
+                    if (kSum) {
+                        // summaries need no scores
+                    } else if (mode == kModeF16) {
+                        const uint64_t dq = kdesc(st + kQ), dk = kdesc(st + kK);
+                        mma4_f16_ss_warp<2, 2>(dp, dq, dk, idesc_p16, 0);
+                        mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
+                    } else if (mode == kModeTF32) {
+                        const uint64_t dqh = dqh0 + (c & 1) * (2 * kTile32 >> 4), dkh = dkh0 + (c & 1) * (2 * kTile32 >> 4);
+                        mma4_tf32_ss_warp(dp, dqh, dkh, idesc_p32, 0);
+                        mma4_tf32_ss_warp(dp, dqh + 512, dkh + 512, idesc_p32, 1);  // (the second 32 columns: 8192 B >> 4)
+                        mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
+                    } else if (lane == 0) {
+                        mbar_arrive(&bars[BAR_PFULL + (c & 1)]);  // exact scores are already in smem
+                    }
+                    __syncwarp();
+                    // U(c) = Kbar^T V (fp16 mode: K^^T V): the k tile read as the MN-major A
+                    const uint64_t dk = mndesc(st + kK), dv = mndesc(st + kV);
+                    const uint32_t du = tmem + kColU + (c & 1) * 64;
+                    mma4_f16_ss_warp<128, 128>(du, dk, dv, idesc_u, 0);
+                    if (kSlices == 2) mma4_f16_ss_warp<128, 128>(tmem + kColO + (c & 1) * 64, dk, mndesc(st + kQ), idesc_u, 0);
+                    mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
+                    su = (su == kSlots - 1) ? 0 : su + 1;
+                    if (z_due) {
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c + 2), ((c + 2) / kSlots) & 1, abort_flag, kWaitLimitNs));
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_z(c + 2);
+                    }
                 }
-            }
-            for (int c = 0; ok && c < G; ++c) {
-                ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
-                if (!ok) break;
-                tc_fence_after();
-                // GP: chunk c + 2's Z reuses the A buffer that gen(c) has read.  It goes before P(c) and
-                // U(c) when the chunk has landed (the gen group forms those gates while it waits for P(c)),
-                // else after them.
-                bool z_due = GP && c + 2 < G;
-                if (z_due && !__any_sync(0xffffffffu, !mbar_test(full(c + 2), ((c + 2) / kSlots) & 1))) {
-                    issue_z(c + 2);
-                    z_due = false;
-                }
-                const uint32_t st = slot0 + su * kSlotBytes;
-                const uint32_t mode = __shfl_sync(0xffffffffu, mode_s[su], 0);
-                const uint32_t dp = tmem + kColP + (c & 1) * 64;
-                if (kSum) {
-                    // summaries need no scores
-                } else if (mode == kModeF16) {
-                    const uint64_t dq = kdesc(st + kQ), dk = kdesc(st + kK);
-                    mma4_f16_ss_warp<2, 2>(dp, dq, dk, idesc_p16, 0);
-                    mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
-                } else if (mode == kModeTF32) {
-                    const uint64_t dqh = dqh0 + (c & 1) * (2 * kTile32 >> 4), dkh = dkh0 + (c & 1) * (2 * kTile32 >> 4);
-                    mma4_tf32_ss_warp(dp, dqh, dkh, idesc_p32, 0);
-                    mma4_tf32_ss_warp(dp, dqh + 512, dkh + 512, idesc_p32, 1);  // (the second 32 columns: 8192 B >> 4)
-                    mma_commit_warp(&bars[BAR_PFULL + (c & 1)]);
-                } else if (lane == 0) {
-                    mbar_arrive(&bars[BAR_PFULL + (c & 1)]);  // exact scores are already in smem
-                }
-                __syncwarp();
-                // U(c) = Kbar^T V (fp16 mode: K^^T V): the k tile read as the MN-major A
-                const uint64_t dk = mndesc(st + kK), dv = mndesc(st + kV);
-                const uint32_t du = tmem + kColU + (c & 1) * 64;
-                mma4_f16_ss_warp<128, 128>(du, dk, dv, idesc_u, 0);
-                if (kSlices == 2) mma4_f16_ss_warp<128, 128>(tmem + kColO + (c & 1) * 64, dk, mndesc(st + kQ), idesc_u, 0);
-                mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
-                su = (su == kSlots - 1) ? 0 : su + 1;
-                if (z_due) {
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(full(c + 2), ((c + 2) / kSlots) & 1, abort_flag, kWaitLimitNs));
+            } else if (!kSum) {
+                const uint32_t idesc_o = instr_desc(kFmtF16, 64, 64, 0, 1);
+                const uint32_t sbuf = smem_u32(smem + kOffS);
+                int so = 0;
+                for (int c = 0; c < G; ++c) {
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_ORDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
                     if (!ok) break;
                     tc_fence_after();
-                    issue_z(c + 2);
+                    // O(c) = Qtil S_[c] + P V  (fp16 mode: Q^ (Diag(c1) S_[c]) + P V); the key
+                    // halves of one real chunk accumulate into the same TMEM buffer
+                    const uint32_t st = slot0 + so * kSlotBytes;
+                    const uint64_t dq = kdesc(st + kQ), ds = mndesc(sbuf + (c & 1) * kTile16);
+                    const uint64_t dpm = kdesc(st + kG), dv = mndesc(st + kV);
+                    const uint32_t d = tmem + kColO + ((c / nh) & 1) * 64;
+                    const uint32_t acc0 = (c % nh) != 0;
+                    mma4_f16_ss_warp<2, 128>(d, dq, ds, idesc_o, acc0);
+                    mma4_f16_ss_warp<2, 128>(d, dpm, dv, idesc_o, 1);
+                    mma_commit2_warp(&bars[BAR_OFULL + (c & 1)], &bars[BAR_EMPTY + so]);  // every product of the slot's chunk is done
+                    so = (so == kSlots - 1) ? 0 : so + 1;
                 }
             }
-        } else if (!kSum) {
-            const uint32_t idesc_o = instr_desc(kFmtF16, 64, 64, 0, 1);
-            const uint32_t sbuf = smem_u32(smem + kOffS);
-            int so = 0;
-            for (int c = 0; c < G; ++c) {
-                ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_ORDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
-                if (!ok) break;
-                tc_fence_after();
-                // O(c) = Qtil S_[c] + P V  (fp16 mode: Q^ (Diag(c1) S_[c]) + P V); the key
-                // halves of one real chunk accumulate into the same TMEM buffer
-                const uint32_t st = slot0 + so * kSlotBytes;
-                const uint64_t dq = kdesc(st + kQ), ds = mndesc(sbuf + (c & 1) * kTile16);
-                const uint64_t dpm = kdesc(st + kG), dv = mndesc(st + kV);
-                const uint32_t d = tmem + kColO + ((c / nh) & 1) * 64;
-                const uint32_t acc0 = (c % nh) != 0;
-                mma4_f16_ss_warp<2, 128>(d, dq, ds, idesc_o, acc0);
-                mma4_f16_ss_warp<2, 128>(d, dpm, dv, idesc_o, 1);
-                mma_commit2_warp(&bars[BAR_OFULL + (c & 1)], &bars[BAR_EMPTY + so]);  // every product of the slot's chunk is done
-                so = (so == kSlots - 1) ? 0 : so + 1;
-            }
+            if (!ok && lane == 0) record_timeout(abort_flag);
+            mma_commit_warp(&bars[BAR_DONE]);  // TMEM is released only after every MMA completed
+            mbar_wait(&bars[BAR_DONE], 0, nullptr, kWaitLimitNs);
         }
-        if (!ok && lane == 0) record_timeout(abort_flag);
-        mma_commit_warp(&bars[BAR_DONE]);  // TMEM is released only after every MMA completed
-        mbar_wait(&bars[BAR_DONE], 0, nullptr, kWaitLimitNs);
-    } else if (warp < 10) {
+    } else if (warp < kEpi0) {
+        if constexpr (kAligned) setmaxnreg_inc<kRegsGen>();
         // ======================================================= gen warpgroups (chunks c = gw mod 2)
-        const int gw = (warp - 2) >> 2;          // 0: even chunks, 1: odd chunks
+        const int gw = (warp - kGen0) >> 2;      // 0: even chunks, 1: odd chunks
         const int bar_id = 1 + gw;
         if constexpr (MODE == kSplitFull) {
             if (gw == 0) named_barrier_sync(kBarSin, 256);  // the epi took the folded start state
@@ -970,7 +984,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         const int row = 16 * q4 + (lane & 15);   // smem row rho of this thread's accumulator row
         const int ch0 = 32 * hc;                 // its 32 key channels (A) / score columns (P)
         const uint32_t lane_base = static_cast<uint32_t>(32 * q4) << 16;
-        const int tg = threadIdx.x - 64 - 128 * gw;
+        const int tg = threadIdx.x - 32 * kGen0 - 128 * gw;
         const int rho_mid = rev ? 32 : 31, rho_last = rev ? 0 : 63;
         // causal mask of this thread's 32 score columns as packed fp16-pair masks (scan order)
         uint32_t vbits = 0u;  // bit s: score column ch0 + s is kept
@@ -1262,6 +1276,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         }
     } else {
         // ======================================================= epi warpgroup (warps 10-13)
+        if constexpr (kAligned) setmaxnreg_inc<kRegsEpi>();
         // Carries the fp32 state of the current key half in registers (thread: channel
         // row, 32 value columns; with two key halves the other half's state waits in So
         // and the two swap after every virtual chunk), writes Diag(c1) S for the readout
@@ -1320,6 +1335,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         // (in the loop it slowed every chunk: the SM's instruction cache is shared by all roles)
         const int cut0 = kBal ? b_chi : G + 1, cut1 = kBal ? b_t0 : G + 1;
         int c = 0;
+        StreamPos cur{};  // chunk c's position (one decode a chunk: the outputs' is the iteration's before)
         // Every epi warp passes the pieces' boundaries, also one that gave up (its warps decide on
         // their own inside the loop): the hand-offs' named barriers then always see all four.
 #pragma unroll 1
@@ -1330,7 +1346,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 // threads' reads after its acquire
                 unsigned long long *f = p.flags + blockIdx.x - 1;
                 bool got = true;
-                if (ok && threadIdx.x == 10 * 32) {
+                if (ok && threadIdx.x == kEpi0 * 32) {
                     got = handoff_wait(f, p.epoch, abort_flag);
                     if (got) *reinterpret_cast<volatile unsigned long long *>(f) = 0ull;
                 }
@@ -1348,10 +1364,11 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             }
             const int c_end = piece == 0 ? cut0 : (piece == 1 ? cut1 : G + 1);
             for (; ok && c < c_end; ++c) {
+                const StreamPos po = cur;  // chunk c - 1
                 if (c < G) {
                     const int sl = c % kSlots, bb = c & 1;
                     const uint32_t ph = (c >> 1) & 1;
-                    const StreamPos ps = pos(c);
+                    const StreamPos ps = cur = pos(c);
                     if (ps.start) {  // a run of a unit starts: its state (every key half)
                         if (kBal && ps.hin) {
                             // S holds the previous CTA's hand-off (taken before this piece)
@@ -1483,7 +1500,6 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         for (int j = 0; j < 8; ++j) ow[8 * hf + j] = Elem<E>::pack(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
                     }
                     tc_fence_before();
-                    const StreamPos po = pos(co);
                     const int b = fdiv(po.bh, p.fd_H), h = po.bh - b * p.H;
                     const int t = walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row);
                     store_row<E, NH == 1 || MODE == kFull>(p, ow, b, h, t, 64 * po.vb + ch0);
@@ -1498,7 +1514,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 // the epi's four warps wrote their rows; one thread fences (for them all, after the
                 // barrier) and sets the flag, so only its warp waits for its stores in flight
                 named_barrier_sync(3, 128);
-                if (threadIdx.x == 10 * 32) {
+                if (threadIdx.x == kEpi0 * 32) {
                     __threadfence();
                     *reinterpret_cast<volatile unsigned long long *>(p.flags + blockIdx.x) = p.epoch;
                 }
