@@ -551,64 +551,70 @@ __device__ __noinline__ void exact_chunk(uint8_t *tq, uint8_t *tk, uint8_t *tgat
 
 // Operands of a tf32-mode chunk (split factors beyond the fp16 range): tf32 Q^ and
 // K^ for the score product in the group's operand buffer, fp16 Qtil = Q^ c1 over q and
-// Kbar = K^ c2 over k.  Re-reads the thread's 32 log-decays from TMEM (A is kept
-// until the operands are built): out of line, this rarer path leaves the fp16 path's
-// code and registers as they are (inlined it cost workload 2 6 %).
+// Kbar = K^ c2 over k.  Re-reads the thread's log-decays from TMEM (A is kept until the operands are
+// built), half of them at a time in a loop: this rarer path is out of line, and what it costs the
+// chunks that take it is its code and the registers its callers lose (GB300, 6,400 tokens: all 32
+// log-decays at once 163 us fp16 and 172 us bf16, two halves in a loop with packed pairs 150 and 159;
+// inlined it cost B = 32, H = 12, 40 x 40 6 %).
 // SUM (summary passes): only Kbar.
 template <typename E, bool SUM>
 __device__ __noinline__ void tf32_operands(uint8_t *tq, uint8_t *tk, uint8_t *opbuf, const float *ref,
                                            uint32_t taddr, int row, int ch0) {
-    uint32_t ar[32];
-    tmem_ld_16x32bx2_x16(taddr + 0, *reinterpret_cast<uint32_t(*)[16]>(&ar[0]));
-    tmem_ld_16x32bx2_x16(taddr + 16, *reinterpret_cast<uint32_t(*)[16]>(&ar[16]));
-    tmem_ld_wait();
     uint8_t *qh = opbuf, *kh = opbuf + kTile32;
+#pragma unroll 1
+    for (int hf = 0; hf < 2; ++hf) {
+        uint32_t ar[16];
+        tmem_ld_16x32bx2_x16(taddr + 16 * hf, ar);
+        tmem_ld_wait();
 #pragma unroll
-    for (int g8 = 0; g8 < 4; ++g8) {
-        const int cl = ch0 + 8 * g8;
-        const uint32_t o16 = sw128(row, cl * 2);
-        const uint4 qw = SUM ? make_uint4(0u, 0u, 0u, 0u) : *reinterpret_cast<const uint4 *>(tq + o16);
-        const uint4 kw = *reinterpret_cast<const uint4 *>(tk + o16);
-        const uint32_t qa[4] = {qw.x, qw.y, qw.z, qw.w}, ka[4] = {kw.x, kw.y, kw.z, kw.w};
-        // A_mid log2, c1 and c2 of the 8 channels (16-byte aligned rows of the references)
-        float am[8], c1v[8], c2v[8];
-        *reinterpret_cast<float4 *>(&am[0]) = *reinterpret_cast<const float4 *>(ref + cl);
-        *reinterpret_cast<float4 *>(&am[4]) = *reinterpret_cast<const float4 *>(ref + cl + 4);
+        for (int g8 = 0; g8 < 2; ++g8) {
+            const int cl = ch0 + 16 * hf + 8 * g8;
+            const uint32_t o16 = sw128(row, cl * 2);
+            const uint4 qw = SUM ? make_uint4(0u, 0u, 0u, 0u) : *reinterpret_cast<const uint4 *>(tq + o16);
+            const uint4 kw = *reinterpret_cast<const uint4 *>(tk + o16);
+            const uint32_t qa[4] = {qw.x, qw.y, qw.z, qw.w}, ka[4] = {kw.x, kw.y, kw.z, kw.w};
+            // A_mid, c1 and c2 of the 8 channels (16-byte aligned rows of the references)
+            f2 am[4], c1v[4], c2v[4];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) am[e] *= kLog2e;
-        *reinterpret_cast<float4 *>(&c1v[0]) = *reinterpret_cast<const float4 *>(ref + 2 * kD + cl);
-        *reinterpret_cast<float4 *>(&c1v[4]) = *reinterpret_cast<const float4 *>(ref + 2 * kD + cl + 4);
-        *reinterpret_cast<float4 *>(&c2v[0]) = *reinterpret_cast<const float4 *>(ref + 3 * kD + cl);
-        *reinterpret_cast<float4 *>(&c2v[4]) = *reinterpret_cast<const float4 *>(ref + 3 * kD + cl + 4);
-        float qs[8], ks[8];
+            for (int e = 0; e < 2; ++e) {
+                const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(ref + cl + 4 * e);
+                const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(ref + 2 * kD + cl + 4 * e);
+                const ulonglong2 c = *reinterpret_cast<const ulonglong2 *>(ref + 3 * kD + cl + 4 * e);
+                am[2 * e] = a.x, am[2 * e + 1] = a.y;
+                c1v[2 * e] = b.x, c1v[2 * e + 1] = b.y;
+                c2v[2 * e] = c.x, c2v[2 * e + 1] = c.y;
+            }
+            f2 q2[4], k2[4];
+            float qs[8], ks[8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 q2 = Elem<E>::unpack(qa[e]), k2 = Elem<E>::unpack(ka[e]);
-            const float e0 = fmaf(__uint_as_float(ar[8 * g8 + 2 * e]), kLog2e, -am[2 * e]);
-            const float e1 = fmaf(__uint_as_float(ar[8 * g8 + 2 * e + 1]), kLog2e, -am[2 * e + 1]);
-            qs[2 * e] = q2.x * ex2(e0);
-            qs[2 * e + 1] = q2.y * ex2(e1);
-            ks[2 * e] = k2.x * ex2(-e0);
-            ks[2 * e + 1] = k2.y * ex2(-e1);
+            for (int e = 0; e < 4; ++e) {
+                const f2 x = fma2(pack2(ar[8 * g8 + 2 * e], ar[8 * g8 + 2 * e + 1]), pack2(kLog2e, kLog2e),
+                                  mul2(am[e], pack2(-kLog2e, -kLog2e)));
+                q2[e] = mul2(Elem<E>::unpack_pair(qa[e]), ex2_pair(x));
+                k2[e] = mul2(Elem<E>::unpack_pair(ka[e]), ex2_neg_pair(x));
+                const float2 a = unpack2(q2[e]), b = unpack2(k2[e]);
+                qs[2 * e] = a.x, qs[2 * e + 1] = a.y;
+                ks[2 * e] = b.x, ks[2 * e + 1] = b.y;
+            }
+            if (!SUM) {
+                *reinterpret_cast<float4 *>(qh + off32(row, cl)) =
+                    make_float4(to_tf32(qs[0]), to_tf32(qs[1]), to_tf32(qs[2]), to_tf32(qs[3]));
+                *reinterpret_cast<float4 *>(qh + off32(row, cl + 4)) =
+                    make_float4(to_tf32(qs[4]), to_tf32(qs[5]), to_tf32(qs[6]), to_tf32(qs[7]));
+                *reinterpret_cast<float4 *>(kh + off32(row, cl)) =
+                    make_float4(to_tf32(ks[0]), to_tf32(ks[1]), to_tf32(ks[2]), to_tf32(ks[3]));
+                *reinterpret_cast<float4 *>(kh + off32(row, cl + 4)) =
+                    make_float4(to_tf32(ks[4]), to_tf32(ks[5]), to_tf32(ks[6]), to_tf32(ks[7]));
+            }
+            uint32_t qo[4], ko[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                qo[e] = h2bits(mul2(q2[e], c1v[e]));
+                ko[e] = h2bits(mul2(k2[e], c2v[e]));
+            }
+            if (!SUM) *reinterpret_cast<uint4 *>(tq + o16) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
+            *reinterpret_cast<uint4 *>(tk + o16) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
         }
-        if (!SUM) {
-            *reinterpret_cast<float4 *>(qh + off32(row, cl)) =
-                make_float4(to_tf32(qs[0]), to_tf32(qs[1]), to_tf32(qs[2]), to_tf32(qs[3]));
-            *reinterpret_cast<float4 *>(qh + off32(row, cl + 4)) =
-                make_float4(to_tf32(qs[4]), to_tf32(qs[5]), to_tf32(qs[6]), to_tf32(qs[7]));
-            *reinterpret_cast<float4 *>(kh + off32(row, cl)) =
-                make_float4(to_tf32(ks[0]), to_tf32(ks[1]), to_tf32(ks[2]), to_tf32(ks[3]));
-            *reinterpret_cast<float4 *>(kh + off32(row, cl + 4)) =
-                make_float4(to_tf32(ks[4]), to_tf32(ks[5]), to_tf32(ks[6]), to_tf32(ks[7]));
-        }
-        uint32_t qo[4], ko[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            qo[e] = h2bits(qs[2 * e] * c1v[2 * e], qs[2 * e + 1] * c1v[2 * e + 1]);
-            ko[e] = h2bits(ks[2 * e] * c2v[2 * e], ks[2 * e + 1] * c2v[2 * e + 1]);
-        }
-        if (!SUM) *reinterpret_cast<uint4 *>(tq + o16) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
-        *reinterpret_cast<uint4 *>(tk + o16) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
     }
 }
 
