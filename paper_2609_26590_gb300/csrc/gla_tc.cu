@@ -1484,7 +1484,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     // the readout of the previous iteration already)
                     if (!kSum && (NH == 2 || kGenOut) && c >= 2)
                         fail = fail || !mbar_wait(&bars[BAR_OFULL + bb], ph ^ 1, abort_flag, kWaitLimitNs);
-                    if (__any_sync(0xffffffffu, fail || *abort_flag != 0u)) {  // the warp leaves together
+                    if (__any_sync(0xffffffffu, fail)) {  // the warp leaves together
                         ok = false;
                         break;
                     }
