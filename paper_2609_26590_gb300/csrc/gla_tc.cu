@@ -115,8 +115,8 @@ enum : uint32_t { kModeF16 = 0, kModeTF32 = 1, kModeExact = 2 };
 enum : int { kFull = 0, kSplitFull = 1, kSummary = 2, kBalanced = 3 };
 constexpr int kMinSegChunks = 2;          // a split segment keeps at least this many chunks
 constexpr int kMaxUnsplitChunks = 5;      // shorter sequences are never split
-constexpr uint32_t kBarSetup = 5;         // named barrier: set-up done
-constexpr uint32_t kBarSin = 4;           // named barrier: epi read the folded start state (ids 1-3: gen groups, epi)
+constexpr uint32_t kBarSetup = 4;         // named barrier: set-up done
+constexpr uint32_t kBarSin = 5;           // named barrier (two key halves): epi read the folded start state
 
 // Shared-memory map (byte offsets from a 1024-aligned base).
 constexpr int kSlotBytes = 4 * kTile16;                        // q @0, k @8K, v @16K, g @24K
@@ -133,6 +133,9 @@ constexpr int kOffRef = kOffW2 + 2 * kW2Bytes;                 // per slot
 constexpr int kOffDecay = kOffRef + kSlots * kRefFloats * 4;   // per slot, 64 fp32
 constexpr int kOffMode = kOffDecay + kSlots * kD * 4;          // per slot u32 mode; 2 x 2 fp32 maxima
 constexpr int kOffBar = kOffMode + 64;
+// the start state's fold (one key half): summaries whose decay products fit the S' buffers; row pitch
+constexpr int kFoldBatch = 32, kFoldPitch = 68;
+static_assert(kSlots >= 4 && 2 * kSlotBytes >= 4 * kD * kD * 4 && kFoldBatch * kD * 4 <= 2 * kTile16, "the fold's ring and coefficients");
 constexpr int kNumBars = 40;
 constexpr int kOffMisc = kOffBar + kNumBars * 8;               // tmem base, abort flag
 constexpr int kSmemBytes = kOffMisc + 64 + 1024;               // + alignment slack
@@ -153,7 +156,8 @@ enum {
     BAR_ZFULL = BAR_OFULL + 2,         // [2] gate producer: Z = a W2 done -> gen
     BAR_GRDY = BAR_ZFULL + 2,          // [2] gate producer: gates G written by the gen group (4) -> A issuer
     BAR_DONE = BAR_GRDY + 2,           // every MMA completed (teardown)
-    BAR_COUNT = BAR_DONE + 1
+    BAR_SIN = BAR_DONE + 1,            // kSplitFull: the epi folded the start state (4) -> producer
+    BAR_COUNT = BAR_SIN + 1
 };
 static_assert(BAR_COUNT <= kNumBars, "barrier space");
 
@@ -438,6 +442,12 @@ __host__ __device__ __forceinline__ bool chunk_walk_start(int order, int T, cons
 __device__ __forceinline__ uint32_t pmask(uint32_t vbits, int e) {
     return (((vbits >> (2 * e)) & 1u) ? 0x0000FFFFu : 0u) | (((vbits >> (2 * e + 1)) & 1u) ? 0xFFFF0000u : 0u);
 }
+
+__device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Spatial token of walk position w (-1 outside the sequence).
 __device__ __forceinline__ int walk_token(int order, int T, const FastDiv &gh, int grid_w, int w) {
@@ -808,6 +818,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             mbar_init(&bars[BAR_ZFULL + i], 1);
             mbar_init(&bars[BAR_GRDY + i], 4);
         }
+        mbar_init(&bars[BAR_SIN], 4);
         mbar_init(&bars[BAR_DONE], 3);  // one commit per issuer warp
         fence_mbar_init();
     }
@@ -834,7 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         }
         fence_proxy_async_smem();
     }
-    // kSplitFull: the start state of the CTA's segment (a split launch gives every CTA one
+    // kSplitFull, two key halves (one: see the epi): the start state of the CTA's segment (a split launch gives every CTA one
     // segment), folded from the summaries of the segments before it by all 512 threads, each
     // taking 8 of a key half's 64 x 64 values and walking the summaries from the latest back
     // (S_start = sum_s' (prod_{s' < s'' < seg} Diag(D_s'')) S_end(s'), Eq. chunk_boundary_main
@@ -842,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     // waited one L2 round trip per summary, about 8 us for the 13th segment.  The result lands in
     // gen warpgroup 0's tf32 operand buffer, which the epi reads on entry; the group writes the
     // buffer only after the epi's arrival on named barrier kBarSin.
-    if constexpr (MODE == kSplitFull) {
+    if constexpr (MODE == kSplitFull && NH == 2) {
         pdl_wait();  // the summaries are the previous grid's: this launch may start before it ends
         const StreamPos p0 = pos(0);
         if (G > 0 && p0.seg > 0) {
@@ -899,6 +910,11 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     const int b = fdiv(ps.bh, p.fd_H), h = ps.bh - b * p.H, c = ps.c;
                     const int xk = 64 * ps.a, xv = 64 * ps.vb;  // channel offsets of the key half, value slice
                     if (!mbar_wait(&bars[BAR_EMPTY + sl], ((g / kSlots) & 1) ^ 1, abort_flag, kWaitLimitNs)) {
+                        record_timeout(abort_flag);
+                        break;
+                    }
+                    // (slots 2 and 3 serve the start state's fold first)
+                    if (MODE == kSplitFull && NH == 1 && g == 2 && ps.seg > 0 && !mbar_wait(&bars[BAR_SIN], 0, abort_flag, kWaitLimitNs)) {
                         record_timeout(abort_flag);
                         break;
                     }
@@ -1076,7 +1092,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         // ======================================================= gen warpgroups (chunks c = gw mod 2)
         const int gw = (warp - kGen0) >> 2;      // 0: even chunks, 1: odd chunks
         const int bar_id = 1 + gw;
-        if constexpr (MODE == kSplitFull) {
+        if constexpr (MODE == kSplitFull && NH == 2) {
             if (gw == 0) named_barrier_sync(kBarSin, 256);  // the epi took the folded start state
         }
         const int q4 = warp & 3, hc = lane >> 4;
@@ -1397,7 +1413,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
 #pragma unroll
             for (int j = 0; j < 16; ++j) So[j] = 0ull;
         }
-        if constexpr (MODE == kSplitFull) {  // the start state the whole CTA folded (segments past the first)
+        if constexpr (MODE == kSplitFull && NH == 2) {  // the start state the whole CTA folded (segments past the first)
             if (G > 0 && pos(0).seg > 0) {
                 const f2 *sin = reinterpret_cast<const f2 *>(smem + kOffOp) + (row * 64 + ch0) / 2;
 #pragma unroll
@@ -1410,29 +1426,96 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             named_barrier_arrive(kBarSin, 256);  // gen warpgroup 0 may now use its operand buffer
         }
         float dp = 1.f, dpo = 1.f;  // summaries: the segment's decay product per key half
-        // Start state of a split sequence's segment seg > 0 (key half `half`): fold the
-        // end states from zero of segments 0 .. seg-1 with their total decays,
-        // S_start(s + 1) = Diag(D_s) S_start(s) + S_end(s).
         const size_t sum_stride = (size_t)kDk * kDv + kDk;
-        auto start_state = [&](f2(&st)[16], int half, const StreamPos &q) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) st[j] = 0ull;
-            const float *base = p.summary + (size_t)q.bh * (p.nseg - 1) * sum_stride;
-            for (int s2 = 0; s2 < q.seg; ++s2, base += sum_stride) {
-                const float d = base[(size_t)kDk * kDv + 64 * half + row];
-                const ulonglong2 *x = reinterpret_cast<const ulonglong2 *>(base + (size_t)(64 * half + row) * kDv + 64 * q.vb + ch0);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const ulonglong2 w = x[j];
-                    st[2 * j] = fma2(pack2(d, d), st[2 * j], w.x);
-                    st[2 * j + 1] = fma2(pack2(d, d), st[2 * j + 1], w.y);
-                }
-            }
-        };
         bool ok = true;
         if (lane == 0) {  // TMEM U buffers start out free: the drains of chunks -2 and -1
             mbar_arrive(&bars[BAR_PURDY + 0]);
             mbar_arrive(&bars[BAR_PURDY + 1]);
+        }
+        // kSplitFull, one key half: the start state of the CTA's segment (a split launch gives every CTA
+        // one segment), folded from the summaries of the segments before it, from the latest back
+        // (S_start = sum_s' (prod_{s' < s'' < seg} Diag(D_s'')) S_end(s'), Eq. chunk_boundary_main across
+        // segments), while the first two chunks load and go through the gen warps: only their S' needs it.
+        // Bound by the L2 reads (16 KB a summary, 64 B a cycle into the SM): cp.async keeps four summaries
+        // in flight, in the slots of chunks 2 and 3, which the producer leaves alone until BAR_SIN.  Each
+        // thread takes the float4s te + 128 j of a summary (rows of whole sectors) and reads back only its
+        // own copies; the products of decays, one row a thread, go through the S' buffers.  GB300, graph
+        // replays, against a fold by all 512 threads before the first chunk: fp16 B = 1, H = 6, 40 x 40 (13
+        // segments) 13.5 -> 11.2 us, with the gate 14.7 -> 12.9; 20 x 20 12.8 -> 10.4; bf16 44 x 44 17.1 ->
+        // 16.4; B = 4, H = 12, 40 x 40 (3 segments of 9 chunks) the same 27.5.
+        if constexpr (MODE == kSplitFull && NH == 1) {
+            const int seg = pos(0).seg;
+            if (seg > 0) {
+                const StreamPos p0 = pos(0);
+                pdl_wait();  // the summaries are the previous grid's: this launch may start before it ends
+                const int te = threadIdx.x - 32 * kEpi0;
+                const int fr = te >> 4, fc = (te & 15) * 4;
+                float *ring = reinterpret_cast<float *>(smem + kOffSlot + 2 * kSlotBytes);  // 4 x [64][64]
+                float *coefs = reinterpret_cast<float *>(smem + kOffS);                     // [kFoldBatch][64]
+                const float *last = p.summary + ((size_t)p0.bh * (p.nseg - 1) + seg - 1) * sum_stride;
+                const float *src = last + (size_t)fr * kDv + 64 * p0.vb + fc, *dec = last + (size_t)kDk * kDv + te;
+                auto fetch = [&](int i) {  // the i-th summary from the latest (one group each, empty past the first)
+                    if (i < seg) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            cp_async_16(ring + (i & 3) * 4096 + (j * 128 + te) * 4, src - i * sum_stride + (size_t)8 * j * kDv);
+                    }
+                    cp_async_commit();
+                };
+#pragma unroll 1
+                for (int i = 0; i < 4; ++i) fetch(i);
+                float4 acc[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                float run = 1.f;  // te < 64: row te's product of the decays so far
+                for (int i0 = 0; i0 < seg; i0 += kFoldBatch) {
+                    const int m = seg - i0 < kFoldBatch ? seg - i0 : kFoldBatch;
+                    if (te < 64) {
+                        for (int i1 = 0; i1 < m; i1 += 8) {
+                            float d[8];
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) d[k] = i1 + k < m ? __ldcg(dec - (i0 + i1 + k) * sum_stride) : 1.f;
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                coefs[(i1 + k) * 64 + te] = run;
+                                run *= d[k];
+                            }
+                        }
+                    }
+                    named_barrier_sync(3, 128);
+#pragma unroll 1
+                    for (int i = 0; i < m; ++i) {
+                        cp_async_wait<3>();
+                        const float *st = ring + ((i0 + i) & 3) * 4096 + te * 4;
+                        const float *cf = coefs + i * 64 + fr;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float4 x = *reinterpret_cast<const float4 *>(st + j * 512);
+                            const float cj = cf[8 * j];
+                            acc[j].x = fmaf(cj, x.x, acc[j].x);
+                            acc[j].y = fmaf(cj, x.y, acc[j].y);
+                            acc[j].z = fmaf(cj, x.z, acc[j].z);
+                            acc[j].w = fmaf(cj, x.w, acc[j].w);
+                        }
+                        fetch(i0 + i + 4);
+                    }
+                    named_barrier_sync(3, 128);  // the coefficients and (last batch) the ring are free
+                }
+                // to the layout of S, through the ring (rows 272 bytes apart: no bank conflicts)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) *reinterpret_cast<float4 *>(ring + (fr + 8 * j) * kFoldPitch + fc) = acc[j];
+                named_barrier_sync(3, 128);
+                const ulonglong2 *sin = reinterpret_cast<const ulonglong2 *>(ring + row * kFoldPitch + ch0);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const ulonglong2 w = sin[j];
+                    S[2 * j] = w.x;
+                    S[2 * j + 1] = w.y;
+                }
+                fence_proxy_async_smem();  // the ring's slots are TMA destinations next
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars[BAR_SIN]);
+            }
         }
         // kBalanced: the loop runs in three pieces (head run, whole units, tail run) with the
         // hand-offs between them, so that the per-chunk loop itself carries no hand-off code
@@ -1483,12 +1566,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
 #pragma unroll
                                 for (int j = 0; j < 16; ++j) So[j] = 0ull;
                             }
-                        } else if constexpr (kSplit) {
-                            if (MODE != kSplitFull || c != 0) {  // (c == 0: S holds the prologue's fold)
-                                start_state(S, 0, ps);
-                                if constexpr (NH == 2) start_state(So, 1, ps);
-                            }
-                        }
+                        }  // (else: a split launch gives every CTA one segment, and S holds the fold)
                         dp = dpo = 1.f;
                     }
                     bool fail = !mbar_wait(&bars[BAR_REFS + sl], (c / kSlots) & 1, abort_flag, kWaitLimitNs);
