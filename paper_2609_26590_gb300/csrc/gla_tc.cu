@@ -2196,10 +2196,13 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     // outputs from the gen warpgroups: fp16 launches of at most one wave (measured on a GB300:
     // +3 to +6 % there; with several units per CTA, or bf16, the epi storing them was faster)
     const bool gen_out = half && tp.n_units <= n_sm;
-    // the output pass of a split starts while its summary pass runs when both fit on the SMs at
-    // once (measured on a GB300: 1.04-1.06x at B = 1, H = 6, 40 x 40, 72 + 78 CTAs; with
-    // 96 + 128 CTAs at B = 2, H = 8, 128 x 128, Dk = Dv = 128, 0.95x)
-    const bool pdl = nseg > 1 && sum_ctas + grid.x <= static_cast<unsigned>(n_sm);
+    // The output pass of a split starts while its summary pass runs (its CTAs start once every summary
+    // CTA has).  One key half: always; CTAs load and prepare their first chunks on SMs as they free up
+    // (GB300, graph replays, pass sizes in CTAs: 96 + 144, B = 4, H = 12, 40 x 40 27.8 -> 26.2 us; 90 + 96
+    // 15.4 -> 14.4; 24 heads of 56 x 56 28.1 -> 26.9; 128 x 128 with 2 heads 26.4 -> 25.5).  Two key halves,
+    // whose CTAs only set up before they wait: when both fit on the SMs at once (90 + 93 CTAs of 44 x 44
+    // 22.0 us against 22.9, 96 + 128 of 128 x 128 the same).
+    const bool pdl = nseg > 1 && (tp.nh == 1 || sum_ctas + grid.x <= static_cast<unsigned>(n_sm));
     if (fuse) {
         if (nseg > 1)
             e = half ? launch_kernel<__half, 1, 1, kSplitFull, true, false, true>(grid, tp, stream, pdl)
