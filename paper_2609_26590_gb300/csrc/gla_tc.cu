@@ -157,7 +157,8 @@ enum {
     BAR_GRDY = BAR_ZFULL + 2,          // [2] gate producer: gates G written by the gen group (4) -> A issuer
     BAR_DONE = BAR_GRDY + 2,           // every MMA completed (teardown)
     BAR_SIN = BAR_DONE + 1,            // kSplitFull: the epi folded the start state (4) -> producer
-    BAR_COUNT = BAR_SIN + 1
+    BAR_GFULL = BAR_SIN + 1,           // [kSlots] gate producer: a (and W2) landed -> Z
+    BAR_COUNT = BAR_GFULL + kSlots
 };
 static_assert(BAR_COUNT <= kNumBars, "barrier space");
 
@@ -805,6 +806,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         *abort_flag = 0u;
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&bars[BAR_FULL + i], 1);
+            mbar_init(&bars[BAR_GFULL + i], 1);
             mbar_init(&bars[BAR_EMPTY + i], MODE == kSummary ? 1 : 2);  // after U(c) and after O(c)
             mbar_init(&bars[BAR_REFS + i], 1);
         }
@@ -925,34 +927,42 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         // buffer of the unit's parity (the unit before last, whose Z products used it,
                         // ended at least four chunks earlier: its last Z completed before this slot freed)
                         const bool w2 = GP && ps.cl == 0;
-                        mbar_arrive_expect_tx(fb, (kSum && kSlices == 1 ? kSlotBytes - kTile16 : kSlotBytes) + (w2 ? kW2Bytes : 0));
-                        if (w2) tma_load_5d(smem + kOffW2 + (fdiv(g, p.fd_L) & 1) * kW2Bytes, &p.w2map, fb, 0, 0, h, 0, 0);
+                        // (the a tile and W2 go first and have their own mbarrier: Z and the gates need nothing
+                        // else; B = 32, H = 12, 40 x 40 bf16 125.5 -> 122.5 us.  The same for loaded gates: 2 to
+                        // 3 % slower at B = 8, H = 16, 80 x 80 and at Dk = Dv = 128, 1 % faster at B = 32)
+                        uint64_t *gb = GP ? &bars[BAR_GFULL + sl] : fb;
+                        if (GP) mbar_arrive_expect_tx(gb, kTile16 + (w2 ? kW2Bytes : 0));
+                        mbar_arrive_expect_tx(fb, GP || (kSum && kSlices == 1) ? kSlotBytes - kTile16 : kSlotBytes);
+                        if (w2) tma_load_5d(smem + kOffW2 + (fdiv(g, p.fd_L) & 1) * kW2Bytes, &p.w2map, gb, 0, 0, h, 0, 0);
                         int x0, y0;
                         if (chunk_walk_start(p.order, p.T, p.fd_gh, c, &x0, &y0)) {
                             // column orders, chunk inside the sequence: one im2col walk per tensor
                             // (boxes per column segment cost the TMA unit one request each and ran
                             // up to 1.9x slower)
+                            if (GP) tma_load_im2col_5d(st + kG, &p.cmaps[T_G], gb, 0, y0, x0, 0, b);
                             if (!kSum) tma_load_im2col_5d(st + kQ, &p.cmaps[T_Q], fb, xk, y0, x0, h, b);
                             tma_load_im2col_5d(st + kK, &p.cmaps[T_K], fb, xk, y0, x0, h, b);
                             tma_load_im2col_5d(st + kV, &p.cmaps[T_V], fb, xv, y0, x0, h, b);
                             if (kSlices == 2) tma_load_im2col_5d(st + kQ, &p.cmaps[T_V], fb, 64, y0, x0, h, b);
-                            tma_load_im2col_5d(st + kG, &p.cmaps[T_G], fb, GP ? 0 : xk, y0, x0, GP ? 0 : h, b);
+                            if (!GP) tma_load_im2col_5d(st + kG, &p.cmaps[T_G], fb, xk, y0, x0, h, b);
                         } else chunk_load_boxes(p.order, p.T, p.fd_gh, p.grid_w, c, [&](int hi, int row, int c2, int c3) {
+                            // gate producer: the 16 projection values of each token, zero-filled to a 128-byte row
+                            if (GP) tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], gb, 0, 0, c2, c3, b);
                             if (!kSum) tma_load_5d(st + kQ + row * 128, &p.maps[T_Q][hi], fb, xk, h, c2, c3, b);
                             tma_load_5d(st + kK + row * 128, &p.maps[T_K][hi], fb, xk, h, c2, c3, b);
                             tma_load_5d(st + kV + row * 128, &p.maps[T_V][hi], fb, xv, h, c2, c3, b);
                             if (kSlices == 2) tma_load_5d(st + kQ + row * 128, &p.maps[T_V][hi], fb, 64, h, c2, c3, b);
-                            // the gate tile, or (gate producer) the 16 projection values of each token,
-                            // zero-filled to a 128-byte row
-                            tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], fb, GP ? 0 : xk, GP ? 0 : h, c2, c3, b);
+                            if (!GP) tma_load_5d(st + kG + row * 128, &p.maps[T_G][hi], fb, xk, h, c2, c3, b);
                         });
                     }
                     ++issued;
                 }
                 if (*abort_flag) {  // never leave while copies are still landing in shared memory
                     for (int g = (issued > kSlots ? issued - kSlots : 0); g < issued; ++g)
-                        if (!(p.drop_load && blockIdx.x == 0 && g == 0))
+                        if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
                             mbar_wait(&bars[BAR_FULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
+                            if (GP) mbar_wait(&bars[BAR_GFULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
+                        }
                 }
             }
         } else {
@@ -1009,7 +1019,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     mma_f16_ss_warp(tmem + kColA + (c & 1) * 64, da, dw, instr_desc(Elem<E>::fmt, 64, 64, 0, 1), 0);
                     mma_commit_warp(&bars[BAR_ZFULL + (c & 1)]);
                 };
-                auto full = [&](int c) -> uint64_t * { return &bars[BAR_FULL + c % kSlots]; };
+                auto full = [&](int c) -> uint64_t * { return &bars[BAR_GFULL + c % kSlots]; };
                 if constexpr (GP) {
                     for (int c = 0; c < 2 && c < G; ++c) {
                         ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, kWaitLimitNs));
@@ -1207,7 +1217,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             const int sl = c % kSlots, bb = c & 1;
             const uint32_t ph = (c >> 1) & 1;
             uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
-            const bool fail = zfail || !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
+            bool fail = zfail || !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
+            // (gate producer: A(c) waited for the a tile only)
+            if constexpr (GP) fail = fail || !mbar_wait(&bars[BAR_FULL + sl], (c / kSlots) & 1, abort_flag, kWaitLimitNs);
             // bf16 values become fp16 MMA operands in place (exact for |v| in the fp16
             // normal range); the loads go first so that their latency hides behind the
             // operand build, the converted words are stored with the operands
