@@ -847,8 +847,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         }
         fence_proxy_async_smem();
     }
-    // kSplitFull, two key halves (one: see the epi): the start state of the CTA's segment (a split launch gives every CTA one
-    // segment), folded from the summaries of the segments before it by all 512 threads, each
+    // kSplitFull, two key halves (one: see the epi): the start state of the CTA's segment (a split
+    // launch gives every CTA one segment), folded from the summaries of the segments before it by all 512 threads, each
     // taking 8 of a key half's 64 x 64 values and walking the summaries from the latest back
     // (S_start = sum_s' (prod_{s' < s'' < seg} Diag(D_s'')) S_end(s'), Eq. chunk_boundary_main
     // across segments) with several summaries' loads in flight.  A serial fold by the epi alone
@@ -1975,9 +1975,9 @@ int pad64(int d) { return (d + 63) / 64 * 64; }
 // SMs splits every sequence into segments of `len` chunks, so that the split
 // launch still fits one wave (units x ceil(N / len) <= SMs).  The split's critical
 // path is the last segment: `len` chunks in each of the two passes, plus the fold
-// of the nseg - 1 earlier summaries into its start state, which the output pass's
-// CTAs do together with many loads in flight.  A graph-replayed sweep of every
-// length on a GB300 (batch-1 and small-batch shapes, 64 <= N <= 256 chunks) fitted
+// of the nseg - 1 earlier summaries into its start state, with several summaries'
+// loads in flight.  A graph-replayed sweep of every length on a GB300, with the fold
+// before the first chunk (batch-1 and small-batch shapes, 64 <= N <= 256 chunks), fitted
 // about 1.95 us per chunk of length against 0.13 us per segment, so the length
 // minimises 15 len + ceil(N / len), at least kMinSegChunks.  Sequences of at most
 // kMaxUnsplitChunks chunks stay whole (5 chunks: 11.4 us whole, 13.4 us split).
