@@ -217,6 +217,11 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float max_nan(float a, float b) {  // NaN when either is (fmaxf drops it)
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
 __device__ __forceinline__ float to_tf32(float x) {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -1263,7 +1268,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             {
                 const float am0 = ref[lane] * kLog2e, al0 = ref[kD + lane] * kLog2e;
                 const float am1 = ref[lane + 32] * kLog2e, al1 = ref[kD + lane + 32] * kLog2e;
-                float m = fmaxf(fmaxf(-am0, am0 - al0), fmaxf(-am1, am1 - al1));
+                // a gate of -inf after the middle leaves A_mid = NaN (0 x -inf in A = L G) and A_last = -inf:
+                // both terms of its channel are NaN, which must not get lost in the maximum
+                float m = max_nan(max_nan(-am0, am0 - al0), max_nan(-am1, am1 - al1));
                 if (!(m <= 3.0e38f)) m = 3.0e38f;  // NaN / inf gates: exact path
                 // (m >= 0 for log gates <= 0, so its bits order like the values.)  One redux instead of five
                 // shuffles and maxima: every warp waits for this, 1.13x at Dk = Dv = 128 and 1.04x at
