@@ -491,13 +491,14 @@ __device__ __forceinline__ void store_row(const TcParams &p, const uint32_t (&ow
         // now pc[q] is the even lane's row and pc[q + 1] the odd lane's, at piece q + odd
         const int other = __shfl_xor_sync(0xffffffffu, t, 1);
         const int t0 = odd ? other : t, t1 = odd ? t : other;
-        const int col = col0 + 8 * odd, ld = p.H * p.Dv;
+        const int col = col0 + 8 * odd;
+        const size_t ld = (size_t)p.H * p.Dv;  // (2^31 elements and more at 2^24 heads)
         E *base = static_cast<E *>(p.out) + ((size_t)b * p.T * p.H + h) * p.Dv + col;
 #pragma unroll
         for (int q = 0; q < 4; q += 2) {
             if (col + 8 * q < p.Dv) {  // (columns past Dv and rows outside the sequence stay behind)
-                if (t0 >= 0) *reinterpret_cast<uint4 *>(base + (size_t)t0 * ld + 8 * q) = pc[q];
-                if (t1 >= 0) *reinterpret_cast<uint4 *>(base + (size_t)t1 * ld + 8 * q) = pc[q + 1];
+                if (t0 >= 0) *reinterpret_cast<uint4 *>(base + t0 * ld + 8 * q) = pc[q];
+                if (t1 >= 0) *reinterpret_cast<uint4 *>(base + t1 * ld + 8 * q) = pc[q + 1];
             }
         }
     } else if (t >= 0) {
