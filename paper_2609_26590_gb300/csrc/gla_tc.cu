@@ -1124,7 +1124,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         // outputs of chunk co (this group's) once O(co) completed: TMEM -> this thread's row at its
         // token's spatial position; false when the wait gave up
         auto gen_out = [&](int co) -> bool {
-            if (!mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs)) return false;
+            // a lane whose wait gave up goes on with the others (what follows is warp-collective) and stores nothing
+            const bool got = mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs);
             tc_fence_after();
             uint32_t r[32];
             tmem_ld_16x32bx2_x16(tmem + lane_base + kColO + (co & 1) * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
@@ -1133,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             uint32_t ow[16];
             const StreamPos po = pos(co);
             const int b = fdiv(po.bh, p.fd_H), h = po.bh - b * p.H;
-            const int t = walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row);
+            const int t = got ? walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row) : -1;
             if constexpr (GATED) {
                 // u = SiLU(r) * o / sqrt(mean_j o_j^2 + eps) * w over the head's Dv outputs: this
                 // thread holds 32 of the row's columns, the lane 16 apart the other 32 (padded
@@ -1169,14 +1170,14 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 for (int j = 0; j < 16; ++j) ow[j] = Elem<E>::pack(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
             }
             store_row<E, true>(p, ow, b, h, t, 64 * po.vb + ch0);
-            return true;
+            return got;
         };
         // GP: chunk cz's gates from Z = a W2 (Sec. 3.1): g = logsigmoid(z + b) / tau in fp32, written as
         // fp16 over the a tile, whose Z product has completed; rows outside the sequence keep g = 0 (no
         // decay), as zero-filled gate rows do.  Done while the group waits for its previous chunk's
         // scores, so that A = L G is ready when that chunk is finished (before, its round trip and the
         // gates stood at the start of every chunk: GB300, B = 32, H = 12, 40 x 40 bf16 182 -> 127 us).
-        auto make_gates = [&](int cz) -> bool {
+        auto make_gates = [&](int cz) {
             const int zb = cz & 1;
             // the position and the bias of the thread's channels first: their loads land while Z does
             // (loaded where they are added, B = 32 127.6 us against 125.9, B = 1, H = 6 fp16 42.4 against 40.4)
@@ -1193,7 +1194,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     bq[2 * q + 1] = __ldg(reinterpret_cast<const ulonglong2 *>(bz + 8 * q + 4));
                 }
             }
-            if (!mbar_wait(&bars[BAR_ZFULL + zb], (cz >> 1) & 1, abort_flag, kWaitLimitNs)) return false;
+            // (a lane whose wait gave up goes on with the others, as the TMEM loads are warp-collective; the
+            // group leaves together at the barrier of its next chunk)
+            if (!mbar_wait(&bars[BAR_ZFULL + zb], (cz >> 1) & 1, abort_flag, kWaitLimitNs)) record_timeout(abort_flag);
             tc_fence_after();
             uint8_t *gt = smem + kOffSlot + (cz % kSlots) * kSlotBytes + kG;
             uint32_t zr[32];
@@ -1214,16 +1217,16 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_GRDY + zb]);  // this warp's rows of G are in smem
-            return true;
         };
-        bool zfail = false;
-        if constexpr (GP) zfail = gw < G && !make_gates(gw);
+        if constexpr (GP) {
+            if (gw < G) make_gates(gw);
+        }
         int last_c = -1;  // the group's last chunk completed (its outputs are stored after the loop)
         for (int c = gw; c < G; c += 2) {
             const int sl = c % kSlots, bb = c & 1;
             const uint32_t ph = (c >> 1) & 1;
             uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
-            bool fail = zfail || !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
+            bool fail = !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
             // (gate producer: A(c) waited for the a tile only)
             if constexpr (GP) fail = fail || !mbar_wait(&bars[BAR_FULL + sl], (c / kSlots) & 1, abort_flag, kWaitLimitNs);
             // bf16 values become fp16 MMA operands in place (exact for |v| in the fp16
@@ -1376,7 +1379,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_PURDY + bb]);  // operands in smem, A(c) read
             if (kSum) continue;  // no scores
-            if constexpr (GP) zfail = c + 2 < G && !make_gates(c + 2);
+            if constexpr (GP) {
+                if (c + 2 < G) make_gates(c + 2);
+            }
             // ---- outputs of the group's previous chunk c-2 (O(c) reuses its TMEM buffer only
             // after ORDY(c), which this group signals below)
             bool ofail = false;
