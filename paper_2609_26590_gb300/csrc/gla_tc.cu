@@ -102,6 +102,7 @@ constexpr int kHeights = 15;              // TMA box heights 1 .. 7, then 8, 16,
 // Rows of the TMA box of height index hi (one tensor map per height).
 __host__ __device__ constexpr int box_height(int hi) { return hi < 7 ? hi + 1 : 8 * (hi - 6); }
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // bounded waits give up after 1 s
+constexpr uint64_t kSlowSummaryNs = 1500000000ull;  // (test hook) longer than that limit
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kGateMinLog2 = -1.0e4f * 1.4426950408889634f;  // g < -1e4 acts as -1e4
 constexpr float kMaxRefF16 = 8.0f;        // fp16 score operands: factors within 2^{+-8}
@@ -184,6 +185,7 @@ struct TcParams {
                                            // [Dk][Dv] and total decay [Dk], fp32
     int drop_load;                         // test hook: CTA 0 withholds its first chunk's load, so the
                                            // bounded waits run out and the call reports a timeout
+    int slow_summary;                      // test hook: CTA 0 of the summary pass starts kSlowSummaryNs late
     unsigned long long *flags;             // kBalanced: per CTA, == epoch once its hand-off state (in
                                            // summary, [64][64] fp32 per CTA) is written; cleared when read
     unsigned long long epoch;              // kBalanced: nonzero, new for every launch
@@ -752,7 +754,13 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     static_assert(kRegsCtl + 2 * kRegsGen + kRegsEpi == 4 * 128, "the registers of the launch");
     // the output pass after a summary pass may start now: its CTAs set up (barriers, TMEM) on
     // the free SMs and wait for this grid only before they read the summaries
-    if constexpr (MODE == kSummary) pdl_launch_dependents();
+    if constexpr (MODE == kSummary) {
+        pdl_launch_dependents();
+        if (p.slow_summary && blockIdx.x == 0) {
+            const uint64_t t0 = global_timer_ns();
+            while (global_timer_ns() - t0 < kSlowSummaryNs) __nanosleep(1000000);
+        }
+    }
     // MODE kFull / kSplitFull: outputs (a split sequence's later segments start from
     // the state folded from the segment summaries).  MODE kSummary: per segment only
     // the end state from zero and the total decay (k, v and gates; no scores or outputs).
@@ -807,6 +815,14 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         return ps;
     };
     const int rev = p.order & 1;
+    // kSplitFull, one key half: the CTA may start long before the summary pass ends, and from its third
+    // chunk on (the readout: from the first) a role's waits depend on the start state the epi folds from
+    // the summaries.  Each role first waits for that grid there (no limit: it ends by itself), so that the
+    // limits of its bounded waits run from then on.  (First segments wait too: they would end early anyway,
+    // and testing for them cost the gen warps registers, 64 heads of 64 x 64 fp16 80.5 us against 79.2.)
+    auto wait_summaries = [&]() {
+        if constexpr (MODE == kSplitFull && NH == 1) pdl_wait();
+    };
 
     if (threadIdx.x == 0) {
         *abort_flag = 0u;
@@ -922,6 +938,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         break;
                     }
                     // (slots 2 and 3 serve the start state's fold first)
+                    if (g == 2) wait_summaries();
                     if (MODE == kSplitFull && NH == 1 && g == 2 && ps.seg > 0 && !mbar_wait(&bars[BAR_SIN], 0, abort_flag, kWaitLimitNs)) {
                         record_timeout(abort_flag);
                         break;
@@ -994,6 +1011,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint64_t dL = kdesc(smem_u32(smem + kOffL));
 
                 for (int c = 0; c < G; ++c) {
+                    if (c == 2) wait_summaries();
                     if constexpr (GP) {
                         // the gen group wrote the chunk's gates (over its a tile, whose Z it has read)
                         ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
@@ -1035,6 +1053,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     }
                 }
                 for (int c = 0; ok && c < G; ++c) {
+                    if (c == 2) wait_summaries();
                     ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
                     if (!ok) break;
                     tc_fence_after();
@@ -1082,6 +1101,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint32_t idesc_o = instr_desc(kFmtF16, 64, 64, 0, 1);
                 const uint32_t sbuf = smem_u32(smem + kOffS);
                 int so = 0;
+                wait_summaries();
                 for (int c = 0; c < G; ++c) {
                     ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_ORDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
                     if (!ok) break;
@@ -1414,6 +1434,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_ORDY + bb]);  // this warp's rows of P are in smem
+            if (last_c < 0) wait_summaries();  // (after the group's first chunk)
             last_c = c;
         }
         if constexpr (kGenOut) {
@@ -1470,9 +1491,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         // 16.4; B = 4, H = 12, 40 x 40 (3 segments of 9 chunks) the same 27.5.
         if constexpr (MODE == kSplitFull && NH == 1) {
             const int seg = pos(0).seg;
+            wait_summaries();  // the summaries are the previous grid's: this launch may start before it ends
             if (seg > 0) {
                 const StreamPos p0 = pos(0);
-                pdl_wait();  // the summaries are the previous grid's: this launch may start before it ends
                 const int te = threadIdx.x - 32 * kEpi0;
                 const int fr = te >> 4, fc = (te & 15) * 4;
                 float *ring = reinterpret_cast<float *>(smem + kOffSlot + 2 * kSlotBytes);  // 4 x [64][64]
@@ -2163,12 +2184,16 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     // test hook for the timeout path (no fault: the data of one chunk simply never arrives)
     const char *drop = std::getenv("GTR_GLA_TEST_DROP_LOAD");
     tp.drop_load = (drop != nullptr && drop[0] == '1') ? 1 : 0;
+    tp.slow_summary = 0;
     const int seqs = static_cast<int>(p.B * p.H) * tp.nv;  // (sequence, value slice) pairs
     const bool half = p.dtype == 1;
     // persistent: one CTA per SM, each walking its share of the work units
     unsigned sum_ctas = 0;
     if (nseg > 1) {  // pass 1: end state from zero and total decay of segments 0 .. nseg-2
         // (two key halves: a unit is one half with every value slice)
+        // test hook for the output pass's waits (that pass starts while this one still runs)
+        const char *slow = std::getenv("GTR_GLA_TEST_SLOW_SUMMARY");
+        tp.slow_summary = (slow != nullptr && slow[0] == '1') ? 1 : 0;
         tp.nsu = nseg - 1;
         tp.fd_nsu = make_fastdiv(tp.nsu);
         tp.n_units = (tp.nh == 2 ? 2 * static_cast<int>(p.B * p.H) : seqs) * tp.nsu;
