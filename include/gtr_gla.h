@@ -147,6 +147,17 @@ size_t gtr_gla_workspace_bytes(int B, int H, int grid_h, int grid_w, int Dk, int
 gtr_status_t gtr_gla_split_plan(int B, int H, int grid_h, int grid_w, int Dk, int Dv, int n_sm,
                                 int *nseg, int *seg_len);
 
+/* The CUDA-core recurrence's launch for these shapes on a device with n_sm SMs
+ * that can place thread-block clusters of up to max_cluster CTAs: *cluster CTAs
+ * share a sequence (0: whole sequences), *columns value columns per CTA.  Host
+ * arithmetic only.  (A launch asks the device which clusters it can place and
+ * takes the largest one at most as large as the rule's, down to whole
+ * sequences.)  Returns GTR_ERR_INVALID_ARG for invalid shapes, n_sm < 1 or NULL
+ * outputs (the outputs are then not written). */
+gtr_status_t gtr_gla_simt_plan(int B, int H, int grid_h, int grid_w, int Dk, int Dv,
+                               gtr_dtype_t dtype, int n_sm, int max_cluster, int *cluster,
+                               int *columns);
+
 /* 1 when the tensor-core schedule balances these shapes on a device with n_sm SMs,
  * else 0 (also for invalid shapes or n_sm < 1).  Balanced: Dk <= 64, no sequence
  * split, more (sequence, 64-column value slice) units than SMs, and a round-robin

@@ -265,6 +265,19 @@ gtr_status_t gtr_gla_split_plan(int B, int H, int grid_h, int grid_w, int Dk, in
     return GTR_OK;
 }
 
+gtr_status_t gtr_gla_simt_plan(int B, int H, int grid_h, int grid_w, int Dk, int Dv, gtr_dtype_t dtype, int n_sm,
+                               int max_cluster, int *cluster, int *columns) {
+    if (!cluster || !columns || n_sm < 1) return GTR_ERR_INVALID_ARG;
+    const gtr_status_t st = check_shape(B, H, grid_h, grid_w, Dk, Dv, 0, dtype);
+    if (st != GTR_OK) return st;
+    const gtr::Problem p{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, B, H, grid_h, grid_w,
+                         Dk, Dv, 0, dtype, (long long)grid_h * grid_w};
+    const gtr::SimtPlan plan = gtr::simt_plan(p, n_sm, max_cluster);
+    *cluster = plan.cluster;
+    *columns = plan.columns;
+    return GTR_OK;
+}
+
 int gtr_gla_balanced_plan(int B, int H, int grid_h, int grid_w, int Dk, int Dv, int n_sm) {
     if (n_sm < 1 || check_shape(B, H, grid_h, grid_w, Dk, Dv, 0, GTR_F16) != GTR_OK || B == 0 || H == 0) return 0;
     gtr::Problem p{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, B, H, grid_h, grid_w,

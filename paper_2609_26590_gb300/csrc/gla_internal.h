@@ -82,6 +82,13 @@ bool tc_gate_supported(const Problem &p, int rank);
 // problem's g pointer is not used).
 cudaError_t launch_tc_gate(const Problem &p, const GateSource &gs, cudaStream_t stream, Ran *ran = nullptr);
 
+// The CUDA-core recurrence's launch on a device with n_sm SMs and clusters of up to max_cluster CTAs.
+struct SimtPlan {
+    int cluster;  // CTAs per sequence (0: whole sequences)
+    int columns;  // value columns per CTA
+};
+SimtPlan simt_plan(const Problem &p, int n_sm, int max_cluster);
+
 // SMs of the current device, looked up once per device.
 cudaError_t sm_count(int *n_sm);
 

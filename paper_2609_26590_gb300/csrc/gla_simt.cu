@@ -580,8 +580,8 @@ __global__ void __launch_bounds__(kSimtThreads, 2) gla_simt_kernel(const __grid_
             }
     }}
 
-// CTAs per sequence: a cluster of 2, 3, 4, 8 or 16 whose groups take a segment each, or 0 for whole
-// sequences, one per group.  The segments cost each token twice (the pass from zero is about half the
+// CTAs per sequence: a cluster of 2, 3, 4, 8 or 16 (at most max_cluster) whose groups take a segment
+// each, or 0 for whole sequences, one per group.  The segments cost each token twice (the pass from zero is about half the
 // work of the one with outputs), so they pay while the launch does not fill the SMs without them: two
 // CTAs fit an SM, and the largest cluster that keeps all CTAs resident measured fastest (GB300, graph
 // replays, Dk = Dv = 64, 1,600 tokens, us at cluster 0 / 2 / 3 / 4 / 8 / 16):
@@ -590,12 +590,43 @@ __global__ void __launch_bounds__(kSimtThreads, 2) gla_simt_kernel(const __grid_
 //    24 sequences  266 / 116 / 82 / 63 / 63 / 84     192 sequences  315 / 337 / 324 / 323 / 344 / 567
 // Clusters of 6 and 12 were slower than 4 and 8 (they fill the GPCs badly), 16 pays only while one
 // CTA an SM is enough.  A segment keeps at least two blocks of tokens.
-int choose_cluster(const Problem &p, int n_sm, int groups) {
+int choose_cluster(const Problem &p, int n_sm, int groups, int max_cluster) {
     const long long units = static_cast<long long>(p.B) * p.H * ((p.Dv + kCols - 1) / kCols);
     const long long blocks = (p.T + kTok - 1) / kTok;
     for (const int c : {16, 8, 4, 3, 2})
-        if (units * c <= (c == kMaxCluster ? 1LL : 2LL) * n_sm && blocks >= 2LL * groups * c) return c;
+        if (c <= max_cluster && units * c <= (c == kMaxCluster ? 1LL : 2LL) * n_sm && blocks >= 2LL * groups * c) return c;
     return 0;
+}
+
+// Whether the current device can place a cluster of `cluster` CTAs of this kernel (one whose GPCs have
+// few SMs, or a context limited to some of them, may not).  Asked once per device, kernel and size.
+template <int DKM, typename E, bool VEC>
+bool cluster_fits(int cluster, int dev) {
+    static std::atomic<unsigned int> known[64] = {}, fits[64] = {};  // a bit per cluster size
+    const unsigned int bit = 1u << cluster;
+    if (dev >= 0 && dev < 64 && (known[dev].load(std::memory_order_acquire) & bit))
+        return (fits[dev].load(std::memory_order_relaxed) & bit) != 0;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(cluster));
+    cfg.blockDim = dim3(kSimtThreads);
+    cfg.dynamicSmemBytes = SimtShape<DKM>::bytes;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gla_simt_kernel<DKM, E, VEC>, &cfg) != cudaSuccess) {
+        n = 0;
+        cudaGetLastError();  // a size the device does not take: the launch falls to a smaller one
+    }
+    if (dev >= 0 && dev < 64) {
+        if (n > 0) fits[dev].fetch_or(bit, std::memory_order_relaxed);
+        known[dev].fetch_or(bit, std::memory_order_release);
+    }
+    return n > 0;
 }
 
 template <int DKM, typename E, bool VEC>
@@ -620,7 +651,8 @@ cudaError_t launch_shape(const Problem &p, cudaStream_t stream) {
     sp.fd_H = make_fastdiv(p.H);
     sp.fd_gh = make_fastdiv(p.grid_h);
     sp.n_seqs = p.B * p.H;
-    const int cluster = choose_cluster(p, n_sm, Sh::G);
+    int cluster = choose_cluster(p, n_sm, Sh::G, kMaxCluster);
+    while (cluster > 0 && !cluster_fits<DKM, E, VEC>(cluster, dev)) cluster = choose_cluster(p, n_sm, Sh::G, cluster - 1);
     const long long blocks = (p.T + kTok - 1) / kTok;
     sp.nseg = cluster > 0 ? cluster * Sh::G : 1;
     sp.seg_len = (blocks + sp.nseg - 1) / sp.nseg * kTok;
@@ -785,6 +817,11 @@ cudaError_t launch_gate_epilogue(const Problem &p, const Gate &gate, cudaStream_
     if (p.dtype == 0) return launch_gate_typed<float>(p, gate, stream);
     if (p.dtype == 1) return launch_gate_typed<__half>(p, gate, stream);
     return launch_gate_typed<__nv_bfloat16>(p, gate, stream);
+}
+
+SimtPlan simt_plan(const Problem &p, int n_sm, int max_cluster) {
+    const int groups = p.Dk <= 32 ? SimtShape<32>::G : p.Dk <= 64 ? SimtShape<64>::G : SimtShape<128>::G;
+    return SimtPlan{choose_cluster(p, n_sm, groups, max_cluster), kCols};
 }
 
 cudaError_t launch_simt(const Problem &p, cudaStream_t stream) {

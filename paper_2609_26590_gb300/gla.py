@@ -65,6 +65,8 @@ def load(path: Optional[str] = None):
         lib.gtr_gla_chunk_walk.argtypes = [ci] * 4 + [ctypes.POINTER(ci)] * 2
         lib.gtr_gla_balanced_walk.restype = ci
         lib.gtr_gla_balanced_walk.argtypes = [ci] * 4 + [ctypes.POINTER(ci), ci, ctypes.POINTER(ci)]
+        lib.gtr_gla_simt_plan.restype = ci
+        lib.gtr_gla_simt_plan.argtypes = [ci] * 9 + [ctypes.POINTER(ci)] * 2
         lib.gtr_gla_split_plan.restype = ci
         lib.gtr_gla_split_plan.argtypes = [ci] * 7 + [ctypes.POINTER(ci)] * 2
         lib.gtr_gla_balanced_plan.restype = ci
@@ -177,6 +179,18 @@ def forward(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, log_gate: torch.T
 def workspace_bytes(B, H, grid_h, grid_w, Dk, Dv, dtype: torch.dtype) -> int:
     """Device workspace ``forward_ws`` needs for these arguments (0: none)."""
     return int(load().gtr_gla_workspace_bytes(B, H, grid_h, grid_w, Dk, Dv, _DTYPES[dtype]))
+
+
+def simt_plan(B: int, H: int, grid_h: int, grid_w: int, Dk: int, Dv: int, dtype: torch.dtype, n_sm: int,
+              max_cluster: int = 16) -> Tuple[int, int]:
+    """(CTAs per sequence, 0 for whole sequences, value columns per CTA) of the CUDA-core recurrence on a
+    device with ``n_sm`` SMs and clusters of up to ``max_cluster`` CTAs, through ``gtr_gla_simt_plan``."""
+    lib = load()
+    cluster, columns = ctypes.c_int(0), ctypes.c_int(0)
+    status = lib.gtr_gla_simt_plan(B, H, grid_h, grid_w, Dk, Dv, _DTYPES[dtype], n_sm, max_cluster,
+                                   ctypes.byref(cluster), ctypes.byref(columns))
+    _check(status, "gtr_gla_simt_plan", lib)
+    return cluster.value, columns.value
 
 
 def split_plan(B: int, H: int, grid_h: int, grid_w: int, Dk: int, Dv: int, n_sm: int) -> Tuple[int, int]:
