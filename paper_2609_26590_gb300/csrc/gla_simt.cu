@@ -572,13 +572,27 @@ __global__ void __launch_bounds__(kSimtThreads, 2) gla_simt_kernel(const __grid_
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int r = row_of(i), col = c0 + col_of(c >> 2) + (c & 3);
-                const float2 x = unpack2(S[i][c]);
-                if (col < Dv && r < Dk) fs[static_cast<long long>(r) * Dv + col] = x.x;
-                if (col < Dv && r + 1 < Dk) fs[static_cast<long long>(r + 1) * Dv + col] = x.y;
+            for (int m = 0; m < 2; ++m) {
+                const int r = row_of(i), col = c0 + col_of(m);
+                const float2 x0 = unpack2(S[i][4 * m]), x1 = unpack2(S[i][4 * m + 1]);
+                const float2 x2 = unpack2(S[i][4 * m + 2]), x3 = unpack2(S[i][4 * m + 3]);
+                float *lo = fs + static_cast<long long>(r) * Dv + col, *hi = lo + Dv;
+                if constexpr (VEC) {  // (Dk and Dv are multiples of four: rows r and r + 1, columns as one)
+                    if (col < Dv && r < Dk) {
+                        *reinterpret_cast<float4 *>(lo) = make_float4(x0.x, x1.x, x2.x, x3.x);
+                        *reinterpret_cast<float4 *>(hi) = make_float4(x0.y, x1.y, x2.y, x3.y);
+                    }
+                } else {
+                    const float xl[4] = {x0.x, x1.x, x2.x, x3.x}, xh[4] = {x0.y, x1.y, x2.y, x3.y};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (col + e < Dv && r < Dk) lo[e] = xl[e];
+                        if (col + e < Dv && r + 1 < Dk) hi[e] = xh[e];
+                    }
+                }
             }
-    }}
+    }
+}
 
 // CTAs per sequence: a cluster of 2, 3, 4, 8 or 16 (at most max_cluster) whose groups take a segment
 // each, or 0 for whole sequences, one per group.  The segments cost each token twice (the pass from zero is about half the
