@@ -594,6 +594,114 @@ __global__ void __launch_bounds__(kSimtThreads, 2) gla_simt_kernel(const __grid_
     }
 }
 
+// Whole sequences in 16 value columns a CTA, for launches that would leave most of the tiles above empty
+// (narrow_columns).  Thread (group, column) owns one column of S over the group's sixteenth of the Dk rows
+// in registers; the readout is sixteen partial sums, added after every block of 16 tokens through shared
+// memory.  Bound by the chain of tokens below about four CTAs an SM, above it by the issue of its
+// broadcast shared-memory reads (three for two rows, against 96 packed operations a read in the tiles).
+constexpr int kNarrowTok = 16, kNarrowCols = 16, kNarrowGroups = 16;
+
+template <int DKM, typename E>
+__global__ void __launch_bounds__(kSimtThreads) gla_simt_narrow_kernel(const __grid_constant__ SimtParams sp) {
+    constexpr int RPT = DKM / kNarrowGroups;               // rows of S per thread
+    constexpr int NQ = kNarrowTok * DKM / kSimtThreads;    // staged q / k / gamma values per thread
+    static_assert(kNarrowTok * kNarrowCols == kSimtThreads, "one staged v value per thread");
+    __shared__ __align__(16) float sq[kNarrowTok][DKM];
+    __shared__ __align__(16) float sk[kNarrowTok][DKM];
+    __shared__ __align__(16) float sgam[kNarrowTok][DKM];
+    __shared__ float sv[kNarrowTok][kNarrowCols];
+    __shared__ float po[kNarrowGroups][kNarrowTok][kNarrowCols];  // partial readouts of the block
+    __shared__ int stok[kNarrowTok];
+
+    const Problem &p = sp.p;
+    const int bh = static_cast<int>(blockIdx.x), b = fdiv(bh, sp.fd_H), h = bh - b * p.H;
+    const int c0 = static_cast<int>(blockIdx.y) * kNarrowCols;
+    const int tid = static_cast<int>(threadIdx.x);
+    const int cj = tid % kNarrowCols, grp = tid / kNarrowCols;  // column and row group owned
+    const int Dk = p.Dk, Dv = p.Dv;
+    const unsigned T = static_cast<unsigned>(p.T);
+    const long long row0 = (static_cast<long long>(b) * p.T) * p.H + h;
+    const E *q = static_cast<const E *>(p.q), *k = static_cast<const E *>(p.k);
+    const E *v = static_cast<const E *>(p.v), *g = static_cast<const E *>(p.g);
+    E *out = static_cast<E *>(p.out);
+
+    // one block's inputs in registers (zeros / gamma = 1 past the sequence and past Dk, Dv:
+    // padding contributes nothing)
+    float rq[NQ], rk[NQ], rg[NQ], rv;
+    int rt = 0;
+    auto load_block = [&](unsigned s0) {
+        const int n = static_cast<int>(T - s0 < kNarrowTok ? T - s0 : kNarrowTok);
+#pragma unroll
+        for (int m = 0; m < NQ; ++m) {
+            const int idx = tid + m * kSimtThreads, j = idx / DKM, i = idx % DKM;
+            float qv = 0.f, kv = 0.f, gam = 1.f;
+            if (j < n && i < Dk) {
+                const long long off = (row0 + static_cast<long long>(scan_token(sp, s0 + j)) * p.H) * Dk + i;
+                qv = to_f32(q[off]);
+                kv = to_f32(k[off]);
+                gam = gamma_of(to_f32(g[off]));
+            }
+            rq[m] = qv;
+            rk[m] = kv;
+            rg[m] = gam;
+        }
+        const int j = tid / kNarrowCols, c = tid % kNarrowCols;
+        rv = 0.f;
+        if (j < n && c0 + c < Dv) rv = to_f32(v[(row0 + static_cast<long long>(scan_token(sp, s0 + j)) * p.H) * Dv + c0 + c]);
+        rt = tid < n ? scan_token(sp, s0 + tid) : 0;
+    };
+
+    float S[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) S[i] = 0.f;
+
+    load_block(0);
+    for (unsigned s0 = 0; s0 < T; s0 += kNarrowTok) {
+        const int n = static_cast<int>(T - s0 < kNarrowTok ? T - s0 : kNarrowTok);
+        __syncthreads();  // the previous block's shared values and partials are consumed
+#pragma unroll
+        for (int m = 0; m < NQ; ++m) {
+            const int idx = tid + m * kSimtThreads;
+            sq[idx / DKM][idx % DKM] = rq[m];
+            sk[idx / DKM][idx % DKM] = rk[m];
+            sgam[idx / DKM][idx % DKM] = rg[m];
+        }
+        sv[tid / kNarrowCols][tid % kNarrowCols] = rv;
+        if (tid < kNarrowTok) stok[tid] = rt;
+        __syncthreads();
+        if (s0 + kNarrowTok < T) load_block(s0 + kNarrowTok);  // in flight while this block runs
+        for (int j = 0; j < n; ++j) {
+            const float vj = sv[j][cj];
+            float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < RPT; i += 2) {
+                const int r = grp * RPT + i;
+                S[i] = fmaf(sgam[j][r], S[i], sk[j][r] * vj);
+                S[i + 1] = fmaf(sgam[j][r + 1], S[i + 1], sk[j][r + 1] * vj);
+                o0 = fmaf(sq[j][r], S[i], o0);
+                o1 = fmaf(sq[j][r + 1], S[i + 1], o1);
+            }
+            po[grp][j][cj] = o0 + o1;
+        }
+        __syncthreads();
+        // the block's outputs: sum over the row groups, scattered to the spatial tokens
+        const int j = tid / kNarrowCols, c = tid % kNarrowCols;
+        if (j < n && c0 + c < Dv) {
+            float o = 0.f;
+#pragma unroll
+            for (int r = 0; r < kNarrowGroups; ++r) o += po[r][j][c];
+            out[(row0 + static_cast<long long>(stok[j]) * p.H) * Dv + c0 + c] = from_f32<E>(o);
+        }
+    }
+    const int col = c0 + cj;
+    if (p.final_state != nullptr && col < Dv) {
+        float *fs = p.final_state + static_cast<long long>(bh) * Dk * Dv;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+            if (grp * RPT + i < Dk) fs[static_cast<long long>(grp * RPT + i) * Dv + col] = S[i];
+    }
+}
+
 // CTAs per sequence: a cluster of 2, 3, 4, 8 or 16 (at most max_cluster) whose groups take a segment
 // each, or 0 for whole sequences, one per group.  The segments cost each token twice (the pass from zero is about half the
 // work of the one with outputs), so they pay while the launch does not fill the SMs without them: two
@@ -610,6 +718,30 @@ int choose_cluster(const Problem &p, int n_sm, int groups, int max_cluster) {
     for (const int c : {16, 8, 4, 3, 2})
         if (c <= max_cluster && units * c <= (c == kMaxCluster ? 1LL : 2LL) * n_sm && blocks >= 2LL * groups * c) return c;
     return 0;
+}
+
+// Whether a launch of whole sequences takes 16 value columns a CTA instead of tiles of 64.  The tiles walk
+// a sequence of up to 32 key channels with one warp, compute all 64 columns however many there are, and
+// take 1 to 2 us longer to start, so they lose (GB300, graph replays, us in tiles / in 16 columns):
+//   Dk <= 32: up to 16 columns at any size (200 sequences of 1,600 tokens at 32 x 16 504 / 300, 2,000 of 256
+//     234 / 193); wider ones while the 16-column CTAs still fit the SMs at once (200 of 1,600 at 32 x 32
+//     533 / 317, 304 of 256 65 / 59; but 400 of 256 at 32 x 32 68 / 89).  At 16 bits twice as far for long
+//     sequences (608 of 1,600 at 32 x 32 935 / 826).
+//   Dk <= 64, up to 16 columns, one SM in two with a second CTA of tiles (400 of 256 at 64 x 16 84 / 75; but 200
+//     45 / 61, 1,000 164 / 178); at 16 bits any number of sequences above that, and long ones (400 of 1,600 694 / 584).
+//   Short sequences in few CTAs (24 of 8 tokens at 64 x 64 4.5 / 3.8, of 32 8.7 / 8.1, at 16 bits 9.9 / 8.8; 1,000 of
+//     16 at 64 x 16 14.2 / 12.1).
+// Above 64 key channels the tiles win (200 of 256 at 128 x 16 78 / 95) but for one or two tokens (4.1 / 3.2).
+bool narrow_columns(const Problem &p, int n_sm) {
+    const long long seqs = static_cast<long long>(p.B) * p.H;
+    const long long ctas = seqs * ((p.Dv + kNarrowCols - 1) / kNarrowCols);
+    const bool half = p.dtype != 0, is_long = p.T >= 1024, one = p.Dv <= kNarrowCols;
+    if (p.Dk > 64) return false;
+    if (p.Dk <= 32) return one || ctas <= (is_long ? (half ? 10LL : 5LL) : (half ? 5LL : 4LL)) * n_sm;
+    if (p.T <= 16 && (one || ctas <= 2LL * n_sm)) return true;
+    if (p.T <= (half ? 48 : 32) && ctas <= n_sm) return true;
+    if (half) return one ? is_long || ctas > 2LL * n_sm : is_long && ctas <= 3LL * n_sm;
+    return one && !is_long && ctas > 2LL * n_sm && ctas <= 3LL * n_sm;
 }
 
 // Whether the current device can place a cluster of `cluster` CTAs of this kernel (one whose GPCs have
@@ -643,6 +775,13 @@ bool cluster_fits(int cluster, int dev) {
     return n > 0;
 }
 
+template <int DKM, typename E>
+cudaError_t launch_narrow(const SimtParams &sp, cudaStream_t stream) {
+    const dim3 grid(static_cast<unsigned>(sp.n_seqs), static_cast<unsigned>((sp.p.Dv + kNarrowCols - 1) / kNarrowCols));
+    gla_simt_narrow_kernel<DKM, E><<<grid, kSimtThreads, 0, stream>>>(sp);
+    return cudaGetLastError();
+}
+
 template <int DKM, typename E, bool VEC>
 cudaError_t launch_shape(const Problem &p, cudaStream_t stream) {
     using Sh = SimtShape<DKM>;
@@ -660,13 +799,16 @@ cudaError_t launch_shape(const Problem &p, cudaStream_t stream) {
             return e;
         set_on_devices.fetch_or(bit);
     }
-    SimtParams sp;
+    SimtParams sp = {};
     sp.p = p;
     sp.fd_H = make_fastdiv(p.H);
     sp.fd_gh = make_fastdiv(p.grid_h);
     sp.n_seqs = p.B * p.H;
     int cluster = choose_cluster(p, n_sm, Sh::G, kMaxCluster);
     while (cluster > 0 && !cluster_fits<DKM, E, VEC>(cluster, dev)) cluster = choose_cluster(p, n_sm, Sh::G, cluster - 1);
+    if constexpr (DKM <= 64) {
+        if (cluster == 0 && narrow_columns(p, n_sm)) return launch_narrow<DKM, E>(sp, stream);
+    }
     const long long blocks = (p.T + kTok - 1) / kTok;
     sp.nseg = cluster > 0 ? cluster * Sh::G : 1;
     sp.seg_len = (blocks + sp.nseg - 1) / sp.nseg * kTok;
@@ -835,7 +977,8 @@ cudaError_t launch_gate_epilogue(const Problem &p, const Gate &gate, cudaStream_
 
 SimtPlan simt_plan(const Problem &p, int n_sm, int max_cluster) {
     const int groups = p.Dk <= 32 ? SimtShape<32>::G : p.Dk <= 64 ? SimtShape<64>::G : SimtShape<128>::G;
-    return SimtPlan{choose_cluster(p, n_sm, groups, max_cluster), kCols};
+    const int cluster = choose_cluster(p, n_sm, groups, max_cluster);
+    return SimtPlan{cluster, cluster == 0 && narrow_columns(p, n_sm) ? kNarrowCols : kCols};
 }
 
 cudaError_t launch_simt(const Problem &p, cudaStream_t stream) {
