@@ -723,25 +723,22 @@ int choose_cluster(const Problem &p, int n_sm, int groups, int max_cluster) {
 // Whether a launch of whole sequences takes 16 value columns a CTA instead of tiles of 64.  The tiles walk
 // a sequence of up to 32 key channels with one warp, compute all 64 columns however many there are, and
 // take 1 to 2 us longer to start, so they lose (GB300, graph replays, us in tiles / in 16 columns):
-//   Dk <= 32: up to 16 columns at any size (200 sequences of 1,600 tokens at 32 x 16 504 / 300, 2,000 of 256
-//     234 / 193); wider ones while the 16-column CTAs still fit the SMs at once (200 of 1,600 at 32 x 32
-//     533 / 317, 304 of 256 65 / 59; but 400 of 256 at 32 x 32 68 / 89).  At 16 bits twice as far for long
-//     sequences (608 of 1,600 at 32 x 32 935 / 826).
-//   Dk <= 64, up to 16 columns, one SM in two with a second CTA of tiles (400 of 256 at 64 x 16 84 / 75; but 200
-//     45 / 61, 1,000 164 / 178); at 16 bits any number of sequences above that, and long ones (400 of 1,600 694 / 584).
-//   Short sequences in few CTAs (24 of 8 tokens at 64 x 64 4.5 / 3.8, of 32 8.7 / 8.1, at 16 bits 9.9 / 8.8; 1,000 of
-//     16 at 64 x 16 14.2 / 12.1).
+//   Dk <= 32: up to 16 columns at any size (200 fp32 sequences of 1,600 tokens at 32 x 16 517 / 234, 2,000 of
+//     256 240 / 151); wider ones up to five 16-column CTAs an SM, at 16 bits eight or, long, twelve (fp32 at
+//     32 x 32: 400 of 256 tokens 75 / 69; fp16 608 of 1,600 954 / 660, but 350 of 256 at 32 x 64 91 / 107).
+//   Dk <= 64: up to 16 columns (fp16 400 of 1,600 at 61 x 14 696 / 453, fp32 1,000 of 16 at 64 x 16 14.1 / 9.8), but
+//     for long fp32 sequences of which the tiles keep one CTA an SM (200 of 1,600 280 / 368; 400 515 / 411);
+//     up to 48 tokens in two CTAs an SM (24 of 32 at 64 x 64 8.7 / 5.8, 60 of 48 11.4 / 10.1; 152 of 32 8.8 / 10.8);
+//     long 16-bit sequences of two column blocks in four (200 of 1,600 at 64 x 32 617 / 449, 350 717 / 870).
 // Above 64 key channels the tiles win (200 of 256 at 128 x 16 78 / 95) but for one or two tokens (4.1 / 3.2).
 bool narrow_columns(const Problem &p, int n_sm) {
-    const long long seqs = static_cast<long long>(p.B) * p.H;
-    const long long ctas = seqs * ((p.Dv + kNarrowCols - 1) / kNarrowCols);
-    const bool half = p.dtype != 0, is_long = p.T >= 1024, one = p.Dv <= kNarrowCols;
+    const long long ctas = static_cast<long long>(p.B) * p.H * ((p.Dv + kNarrowCols - 1) / kNarrowCols);
+    const bool half = p.dtype != 0, one = p.Dv <= kNarrowCols;
     if (p.Dk > 64) return false;
-    if (p.Dk <= 32) return one || ctas <= (is_long ? (half ? 10LL : 5LL) : (half ? 5LL : 4LL)) * n_sm;
-    if (p.T <= 16 && (one || ctas <= 2LL * n_sm)) return true;
-    if (p.T <= (half ? 48 : 32) && ctas <= n_sm) return true;
-    if (half) return one ? is_long || ctas > 2LL * n_sm : is_long && ctas <= 3LL * n_sm;
-    return one && !is_long && ctas > 2LL * n_sm && ctas <= 3LL * n_sm;
+    if (p.Dk <= 32) return one || ctas <= (half ? (p.T >= 1024 ? 12LL : 8LL) : 5LL) * n_sm;
+    if (one) return half || p.T <= 256 || ctas > 2LL * n_sm;
+    if (p.T <= 48) return ctas <= 2LL * n_sm;
+    return half && p.T >= 1024 && p.Dv <= 2 * kNarrowCols && ctas <= 4LL * n_sm;
 }
 
 // Whether the current device can place a cluster of `cluster` CTAs of this kernel (one whose GPCs have

@@ -50,17 +50,19 @@ def test_falls_to_smaller_clusters(max_cluster):
             assert got == rule(*shape, n_sm, max_cluster) and (got == 0 or got <= max_cluster)
 
 
-# whole sequences (no cluster): 16 columns a CTA for narrow values, up to 32 key channels while those
-# CTAs fit the SMs at once, and short sequences; tiles of 64 columns otherwise
+# whole sequences (no cluster): 16 columns a CTA for narrow values, for up to 32 key channels while those
+# CTAs are few, for short sequences and for long 16-bit ones; tiles of 64 columns otherwise
 COLUMNS = [
-    ((1, 200, 40, 40, 32, 16), "f32", 16), ((1, 4000, 16, 16, 32, 16), "f32", 16), ((1, 200, 40, 40, 32, 17), "f32", 16),
-    ((1, 380, 40, 40, 32, 32), "f32", 16), ((1, 381, 40, 40, 32, 32), "f32", 64), ((1, 400, 16, 16, 32, 32), "f32", 64),
-    ((1, 400, 40, 40, 20, 20), "f16", 16), ((1, 400, 16, 16, 20, 20), "f16", 64), ((1, 761, 40, 40, 20, 20), "f16", 64),
-    ((1, 304, 16, 16, 64, 16), "f32", 64), ((1, 305, 16, 16, 64, 16), "f32", 16), ((1, 456, 16, 16, 64, 16), "f32", 16),
-    ((1, 457, 16, 16, 64, 16), "f32", 64), ((1, 400, 40, 40, 64, 16), "f32", 64), ((1, 400, 40, 40, 61, 14), "f16", 16),
-    ((1, 153, 40, 40, 61, 20), "f16", 16), ((1, 400, 40, 40, 61, 20), "f16", 64), ((1, 400, 40, 40, 64, 64), "f32", 64),
-    ((1, 24, 2, 4, 64, 64), "f32", 16), ((1, 24, 4, 8, 64, 64), "f32", 16), ((1, 24, 5, 8, 64, 64), "f32", 64),
-    ((1, 24, 5, 8, 64, 64), "f16", 16), ((1, 400, 16, 16, 65, 16), "f32", 64),
+    ((1, 200, 40, 40, 32, 16), "f32", 16), ((1, 4000, 16, 16, 32, 16), "f32", 16),
+    ((1, 380, 16, 16, 32, 17), "f32", 16), ((1, 381, 16, 16, 32, 17), "f32", 64),
+    ((1, 912, 40, 40, 20, 20), "f16", 16), ((1, 913, 40, 40, 20, 20), "f16", 64),
+    ((1, 608, 16, 16, 20, 20), "f16", 16), ((1, 609, 16, 16, 20, 20), "f16", 64),
+    ((1, 304, 16, 16, 33, 16), "f32", 16), ((1, 304, 16, 17, 64, 16), "f32", 64), ((1, 305, 16, 17, 64, 16), "f32", 16),
+    ((1, 304, 40, 40, 61, 14), "f16", 16), ((1, 400, 16, 16, 65, 16), "f32", 64),
+    ((1, 24, 6, 8, 64, 64), "f32", 16), ((1, 76, 6, 8, 64, 64), "f32", 16), ((1, 77, 6, 8, 64, 64), "f32", 64),
+    ((1, 24, 7, 7, 64, 64), "f32", 64),
+    ((1, 304, 32, 32, 61, 20), "f16", 16), ((1, 305, 32, 32, 61, 20), "f16", 64), ((1, 200, 32, 32, 61, 33), "f16", 64),
+    ((1, 200, 31, 33, 61, 20), "f16", 64), ((1, 200, 32, 32, 61, 20), "f32", 64), ((1, 400, 40, 40, 64, 64), "f32", 64),
 ]
 
 
