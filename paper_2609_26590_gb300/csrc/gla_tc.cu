@@ -102,7 +102,7 @@ constexpr int kHeights = 15;              // TMA box heights 1 .. 7, then 8, 16,
 // Rows of the TMA box of height index hi (one tensor map per height).
 __host__ __device__ constexpr int box_height(int hi) { return hi < 7 ? hi + 1 : 8 * (hi - 6); }
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // bounded waits give up after 1 s
-constexpr uint64_t kSlowSummaryNs = 1500000000ull;  // (test hook) longer than that limit
+constexpr uint64_t kSlowLoadNs = 800000000ull;    // (test hook) less than that limit, twice it more
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kGateMinLog2 = -1.0e4f * 1.4426950408889634f;  // g < -1e4 acts as -1e4
 constexpr float kMaxRefF16 = 8.0f;        // fp16 score operands: factors within 2^{+-8}
@@ -183,9 +183,9 @@ struct TcParams {
     int nsu;                               // segments per (sequence, value slice) among this launch's units
     float *summary;                        // nseg > 1: per (sequence, segment < nseg - 1) end state from zero
                                            // [Dk][Dv] and total decay [Dk], fp32
-    int drop_load;                         // test hook: CTA 0 withholds its first chunk's load, so the
-                                           // bounded waits run out and the call reports a timeout
-    int slow_summary;                      // test hook: CTA 0 of the summary pass starts kSlowSummaryNs late
+    int drop_load;                         // test hook, 1: CTA 0 withholds its first chunk's load, so the
+                                           // bounded waits run out and the call reports a timeout; 2: CTA 0
+                                           // of the summary pass loads two of its chunks kSlowLoadNs late
     unsigned long long *flags;             // kBalanced: per CTA, == epoch once its hand-off state (in
                                            // summary, [64][64] fp32 per CTA) is written; cleared when read
     unsigned long long epoch;              // kBalanced: nonzero, new for every launch
@@ -754,13 +754,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     static_assert(kRegsCtl + 2 * kRegsGen + kRegsEpi == 4 * 128, "the registers of the launch");
     // the output pass after a summary pass may start now: its CTAs set up (barriers, TMEM) on
     // the free SMs and wait for this grid only before they read the summaries
-    if constexpr (MODE == kSummary) {
-        pdl_launch_dependents();
-        if (p.slow_summary && blockIdx.x == 0) {
-            const uint64_t t0 = global_timer_ns();
-            while (global_timer_ns() - t0 < kSlowSummaryNs) __nanosleep(1000000);
-        }
-    }
+    if constexpr (MODE == kSummary) pdl_launch_dependents();
     // MODE kFull / kSplitFull: outputs (a split sequence's later segments start from
     // the state folded from the segment summaries).  MODE kSummary: per segment only
     // the end state from zero and the total decay (k, v and gates; no scores or outputs).
@@ -945,7 +939,11 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     }
                     uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
                     uint64_t *fb = &bars[BAR_FULL + sl];
-                    if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
+                    if (kSum && p.drop_load == 2 && blockIdx.x == 0 && (g == 0 || g == 2)) {
+                        const uint64_t t0 = global_timer_ns();
+                        while (global_timer_ns() - t0 < kSlowLoadNs) __nanosleep(1000000);
+                    }
+                    if (!(p.drop_load == 1 && blockIdx.x == 0 && g == 0)) {
                         // gate producer: a unit's first chunk also brings the head's W2 block, into the
                         // buffer of the unit's parity (the unit before last, whose Z products used it,
                         // ended at least four chunks earlier: its last Z completed before this slot freed)
@@ -982,7 +980,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 }
                 if (*abort_flag) {  // never leave while copies are still landing in shared memory
                     for (int g = (issued > kSlots ? issued - kSlots : 0); g < issued; ++g)
-                        if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
+                        if (!(p.drop_load == 1 && blockIdx.x == 0 && g == 0)) {
                             mbar_wait(&bars[BAR_FULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
                             if (GP) mbar_wait(&bars[BAR_GFULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
                         }
@@ -2181,19 +2179,15 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.summary = static_cast<float *>(workspace);
     tp.flags = nullptr;
     tp.epoch = 0;
-    // test hook for the timeout path (no fault: the data of one chunk simply never arrives)
+    // test hook for the timeout path (no fault: the data of one chunk simply never arrives, or late)
     const char *drop = std::getenv("GTR_GLA_TEST_DROP_LOAD");
-    tp.drop_load = (drop != nullptr && drop[0] == '1') ? 1 : 0;
-    tp.slow_summary = 0;
+    tp.drop_load = drop == nullptr ? 0 : drop[0] == '1' ? 1 : drop[0] == '2' ? 2 : 0;
     const int seqs = static_cast<int>(p.B * p.H) * tp.nv;  // (sequence, value slice) pairs
     const bool half = p.dtype == 1;
     // persistent: one CTA per SM, each walking its share of the work units
     unsigned sum_ctas = 0;
     if (nseg > 1) {  // pass 1: end state from zero and total decay of segments 0 .. nseg-2
         // (two key halves: a unit is one half with every value slice)
-        // test hook for the output pass's waits (that pass starts while this one still runs)
-        const char *slow = std::getenv("GTR_GLA_TEST_SLOW_SUMMARY");
-        tp.slow_summary = (slow != nullptr && slow[0] == '1') ? 1 : 0;
         tp.nsu = nseg - 1;
         tp.fd_nsu = make_fastdiv(tp.nsu);
         tp.n_units = (tp.nh == 2 ? 2 * static_cast<int>(p.B * p.H) : seqs) * tp.nsu;
