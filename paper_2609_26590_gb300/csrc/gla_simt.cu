@@ -850,7 +850,7 @@ __global__ void __launch_bounds__(256) gate_epilogue_kernel(E *out, const E *r, 
     const int lane = threadIdx.x & 31;
     E *o_row = out + row * Dv;
     const E *r_row = r + row * Dv;
-    float o[8];
+    float o[4];
     float ss = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {

@@ -1462,10 +1462,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const f2 *sin = reinterpret_cast<const f2 *>(smem + kOffOp) + (row * 64 + ch0) / 2;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) S[j] = sin[j];
-                if constexpr (NH == 2) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) So[j] = sin[64 * 32 + j];
-                }
+                for (int j = 0; j < 16; ++j) So[j] = sin[64 * 32 + j];
             }
             named_barrier_arrive(kBarSin, 256);  // gen warpgroup 0 may now use its operand buffer
         }
