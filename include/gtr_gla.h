@@ -386,8 +386,8 @@ gtr_status_t gtr_gla_fwd_host(const void *q_host, const void *k_host, const void
  * call reports GTR_ERR_TIMEOUT (no fault is involved).  A split call's summary
  * pass may take longer than that limit without a timeout: the waits of its
  * output pass that depend on it start once it has ended.  Test hook for that:
- * GTR_GLA_TEST_DROP_LOAD=2 makes the summary pass's first CTA load two of its
- * chunks 0.8 s late each; the call's results stay the same. */
+ * GTR_GLA_TEST_DROP_LOAD=2 launches a grid that takes 1.5 s between the two
+ * passes; the call's results stay the same. */
 gtr_status_t gtr_gla_sync_status(cudaStream_t stream);
 
 /* Schedules a forward call can run (gtr_gla_last_schedule). */

@@ -102,7 +102,6 @@ constexpr int kHeights = 15;              // TMA box heights 1 .. 7, then 8, 16,
 // Rows of the TMA box of height index hi (one tensor map per height).
 __host__ __device__ constexpr int box_height(int hi) { return hi < 7 ? hi + 1 : 8 * (hi - 6); }
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // bounded waits give up after 1 s
-constexpr uint64_t kSlowLoadNs = 800000000ull;    // (test hook) less than that limit, twice it more
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kGateMinLog2 = -1.0e4f * 1.4426950408889634f;  // g < -1e4 acts as -1e4
 constexpr float kMaxRefF16 = 8.0f;        // fp16 score operands: factors within 2^{+-8}
@@ -183,9 +182,8 @@ struct TcParams {
     int nsu;                               // segments per (sequence, value slice) among this launch's units
     float *summary;                        // nseg > 1: per (sequence, segment < nseg - 1) end state from zero
                                            // [Dk][Dv] and total decay [Dk], fp32
-    int drop_load;                         // test hook, 1: CTA 0 withholds its first chunk's load, so the
-                                           // bounded waits run out and the call reports a timeout; 2: CTA 0
-                                           // of the summary pass loads two of its chunks kSlowLoadNs late
+    int drop_load;                         // test hook: CTA 0 withholds its first chunk's load, so the
+                                           // bounded waits run out and the call reports a timeout
     unsigned long long *flags;             // kBalanced: per CTA, == epoch once its hand-off state (in
                                            // summary, [64][64] fp32 per CTA) is written; cleared when read
     unsigned long long epoch;              // kBalanced: nonzero, new for every launch
@@ -939,11 +937,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     }
                     uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
                     uint64_t *fb = &bars[BAR_FULL + sl];
-                    if (kSum && p.drop_load == 2 && blockIdx.x == 0 && (g == 0 || g == 2)) {
-                        const uint64_t t0 = global_timer_ns();
-                        while (global_timer_ns() - t0 < kSlowLoadNs) __nanosleep(1000000);
-                    }
-                    if (!(p.drop_load == 1 && blockIdx.x == 0 && g == 0)) {
+                    if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
                         // gate producer: a unit's first chunk also brings the head's W2 block, into the
                         // buffer of the unit's parity (the unit before last, whose Z products used it,
                         // ended at least four chunks earlier: its last Z completed before this slot freed)
@@ -980,7 +974,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 }
                 if (*abort_flag) {  // never leave while copies are still landing in shared memory
                     for (int g = (issued > kSlots ? issued - kSlots : 0); g < issued; ++g)
-                        if (!(p.drop_load == 1 && blockIdx.x == 0 && g == 0)) {
+                        if (!(p.drop_load && blockIdx.x == 0 && g == 0)) {
                             mbar_wait(&bars[BAR_FULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
                             if (GP) mbar_wait(&bars[BAR_GFULL + g % kSlots], (g / kSlots) & 1, nullptr, kWaitLimitNs);
                         }
@@ -1141,9 +1135,10 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             if (rev ? (ch0 + s >= row) : (ch0 + s <= row)) vbits |= 1u << s;
         // outputs of chunk co (this group's) once O(co) completed: TMEM -> this thread's row at its
         // token's spatial position; false when the wait gave up
-        auto gen_out = [&](int co) -> bool {
-            // a lane whose wait gave up goes on with the others (what follows is warp-collective) and stores nothing
-            const bool got = mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs);
+        auto gen_out = [&](int co) {
+            // (a lane whose wait gave up goes on with the others, as what follows is warp-collective; the group
+            // leaves together at the barrier of its next chunk, and the outputs are then undefined)
+            if (!mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs)) record_timeout(abort_flag);
             tc_fence_after();
             uint32_t r[32];
             tmem_ld_16x32bx2_x16(tmem + lane_base + kColO + (co & 1) * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
@@ -1152,7 +1147,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             uint32_t ow[16];
             const StreamPos po = pos(co);
             const int b = fdiv(po.bh, p.fd_H), h = po.bh - b * p.H;
-            const int t = got ? walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row) : -1;
+            const int t = walk_token(p.order, p.T, p.fd_gh, p.grid_w, chunk_w0(p.order, p.T, po.c) + row);
             if constexpr (GATED) {
                 // u = SiLU(r) * o / sqrt(mean_j o_j^2 + eps) * w over the head's Dv outputs: this
                 // thread holds 32 of the row's columns, the lane 16 apart the other 32 (padded
@@ -1188,7 +1183,6 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 for (int j = 0; j < 16; ++j) ow[j] = Elem<E>::pack(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
             }
             store_row<E, true>(p, ow, b, h, t, 64 * po.vb + ch0);
-            return got;
         };
         // GP: chunk cz's gates from Z = a W2 (Sec. 3.1): g = logsigmoid(z + b) / tau in fp32, written as
         // fp16 over the a tile, whose Z product has completed; rows outside the sequence keep g = 0 (no
@@ -1402,14 +1396,13 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             }
             // ---- outputs of the group's previous chunk c-2 (O(c) reuses its TMEM buffer only
             // after ORDY(c), which this group signals below)
-            bool ofail = false;
             if constexpr (kGenOut) {
-                if (c >= 2) ofail = !gen_out(c - 2);
+                if (c >= 2) gen_out(c - 2);
             }
             // ---- masked scores of chunk c over its gate tile (consumed by A(c) long ago)
             // (a warp that gives up here skips the rest of the chunk; the group leaves together at
             // the barrier of its next one)
-            const bool pfail = ofail || !mbar_wait(&bars[BAR_PFULL + bb], ph, abort_flag, kWaitLimitNs);
+            const bool pfail = !mbar_wait(&bars[BAR_PFULL + bb], ph, abort_flag, kWaitLimitNs);
             if (__any_sync(0xffffffffu, pfail)) {
                 if (lane == 0) record_timeout(abort_flag);
                 continue;
@@ -1436,7 +1429,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             last_c = c;
         }
         if constexpr (kGenOut) {
-            if (last_c >= 0 && last_c + 2 >= G && !gen_out(last_c)) record_timeout(abort_flag);
+            if (last_c >= 0 && last_c + 2 >= G) gen_out(last_c);
         }
     } else {
         // ======================================================= epi warpgroup (warps 10-13)
@@ -1753,6 +1746,14 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
+}
+
+// Test hook: launched between a split's passes, it stands for a summary pass that takes longer than the
+// limit of the bounded waits: the output pass starts while it runs and waits for it.
+__global__ void slow_grid_kernel() {
+    pdl_launch_dependents();
+    const uint64_t t0 = global_timer_ns();
+    while (global_timer_ns() - t0 < kWaitLimitNs + kWaitLimitNs / 2) __nanosleep(1000000);
 }
 
 // ---------------------------------------------------------------- host side
@@ -2177,9 +2178,10 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.summary = static_cast<float *>(workspace);
     tp.flags = nullptr;
     tp.epoch = 0;
-    // test hook for the timeout path (no fault: the data of one chunk simply never arrives, or late)
+    // test hooks: 1, the timeout path (no fault: the data of one chunk simply never arrives); 2, a slow
+    // grid between a split's passes
     const char *drop = std::getenv("GTR_GLA_TEST_DROP_LOAD");
-    tp.drop_load = drop == nullptr ? 0 : drop[0] == '1' ? 1 : drop[0] == '2' ? 2 : 0;
+    tp.drop_load = (drop != nullptr && drop[0] == '1') ? 1 : 0;
     const int seqs = static_cast<int>(p.B * p.H) * tp.nv;  // (sequence, value slice) pairs
     const bool half = p.dtype == 1;
     // persistent: one CTA per SM, each walking its share of the work units
@@ -2194,6 +2196,7 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
         sum_ctas = grid.x;
         e = half ? launch_shape<__half, kSummary>(grid, tp, stream) : launch_shape<__nv_bfloat16, kSummary>(grid, tp, stream);
         if (e != cudaSuccess) return e;
+        if (drop != nullptr && drop[0] == '2') slow_grid_kernel<<<1, 32, 0, stream>>>();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     tp.nsu = nseg;
