@@ -383,11 +383,11 @@ gtr_status_t gtr_gla_fwd_host(const void *q_host, const void *k_host, const void
  * the context stays usable (the outputs of that call are undefined).  Test
  * hook for this path: with the environment variable GTR_GLA_TEST_DROP_LOAD=1
  * the tensor-core schedule withholds one chunk's load in its first CTA, so the
- * call reports GTR_ERR_TIMEOUT (no fault is involved).  A split call's summary
- * pass may take longer than that limit without a timeout: the waits of its
- * output pass that depend on it start once it has ended.  Test hook for that:
- * GTR_GLA_TEST_DROP_LOAD=2 launches a grid that takes 1.5 s between the two
- * passes; the call's results stay the same. */
+ * call reports GTR_ERR_TIMEOUT (no fault is involved).  The output pass of a
+ * split call starts while its summary pass runs, and its waits allow 0.1 ms per
+ * chunk of a segment more for that.  Test hook for it: GTR_GLA_TEST_DROP_LOAD=2
+ * launches a grid between the two passes that takes 1 s and half of that
+ * allowance; the call's results stay the same. */
 gtr_status_t gtr_gla_sync_status(cudaStream_t stream);
 
 /* Schedules a forward call can run (gtr_gla_last_schedule). */

@@ -102,6 +102,9 @@ constexpr int kHeights = 15;              // TMA box heights 1 .. 7, then 8, 16,
 // Rows of the TMA box of height index hi (one tensor map per height).
 __host__ __device__ constexpr int box_height(int hi) { return hi < 7 ? hi + 1 : 8 * (hi - 6); }
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // bounded waits give up after 1 s
+// what a chunk of a summary pass may take, on top of that, for the output pass that waits for it: ten times
+// what the slowest ones (all scores exact) take
+constexpr uint64_t kSummaryChunkNs = 100000ull;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kGateMinLog2 = -1.0e4f * 1.4426950408889634f;  // g < -1e4 acts as -1e4
 constexpr float kMaxRefF16 = 8.0f;        // fp16 score operands: factors within 2^{+-8}
@@ -184,6 +187,7 @@ struct TcParams {
                                            // [Dk][Dv] and total decay [Dk], fp32
     int drop_load;                         // test hook: CTA 0 withholds its first chunk's load, so the
                                            // bounded waits run out and the call reports a timeout
+    unsigned long long wait_limit;         // kSplitFull, one key half: the bounded waits' limit in ns
     unsigned long long *flags;             // kBalanced: per CTA, == epoch once its hand-off state (in
                                            // summary, [64][64] fp32 per CTA) is written; cleared when read
     unsigned long long epoch;              // kBalanced: nonzero, new for every launch
@@ -807,14 +811,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         return ps;
     };
     const int rev = p.order & 1;
-    // kSplitFull, one key half: the CTA may start long before the summary pass ends, and from its third
-    // chunk on (the readout: from the first) a role's waits depend on the start state the epi folds from
-    // the summaries.  Each role first waits for that grid there (no limit: it ends by itself), so that the
-    // limits of its bounded waits run from then on.  (First segments wait too: they would end early anyway,
-    // and testing for them cost the gen warps registers, 64 heads of 64 x 64 fp16 80.5 us against 79.2.)
-    auto wait_summaries = [&]() {
-        if constexpr (MODE == kSplitFull && NH == 1) pdl_wait();
-    };
+    // kSplitFull, one key half: the CTA may start long before the summary pass ends, and in segments past
+    // the first its roles' waits depend on the start state the epi folds from the summaries (from the third
+    // chunk on; the readout: from the first).  So their limit is the launch's: 1 s and the time that pass
+    // may take at most.  (Waiting for the grid in every role, or a limit that starts when the epi has seen
+    // it end, cost 0.1 to 0.5 us of an 11 us call and 2 % of 80 us ones.)
+    const uint64_t limit = MODE == kSplitFull && NH == 1 ? p.wait_limit : kWaitLimitNs;
 
     if (threadIdx.x == 0) {
         *abort_flag = 0u;
@@ -925,13 +927,12 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     const StreamPos ps = pos(g);
                     const int b = fdiv(ps.bh, p.fd_H), h = ps.bh - b * p.H, c = ps.c;
                     const int xk = 64 * ps.a, xv = 64 * ps.vb;  // channel offsets of the key half, value slice
-                    if (!mbar_wait(&bars[BAR_EMPTY + sl], ((g / kSlots) & 1) ^ 1, abort_flag, kWaitLimitNs)) {
+                    if (!mbar_wait(&bars[BAR_EMPTY + sl], ((g / kSlots) & 1) ^ 1, abort_flag, limit)) {
                         record_timeout(abort_flag);
                         break;
                     }
                     // (slots 2 and 3 serve the start state's fold first)
-                    if (g == 2) wait_summaries();
-                    if (MODE == kSplitFull && NH == 1 && g == 2 && ps.seg > 0 && !mbar_wait(&bars[BAR_SIN], 0, abort_flag, kWaitLimitNs)) {
+                    if (MODE == kSplitFull && NH == 1 && g == 2 && ps.seg > 0 && !mbar_wait(&bars[BAR_SIN], 0, abort_flag, limit)) {
                         record_timeout(abort_flag);
                         break;
                     }
@@ -1003,17 +1004,16 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint64_t dL = kdesc(smem_u32(smem + kOffL));
 
                 for (int c = 0; c < G; ++c) {
-                    if (c == 2) wait_summaries();
                     if constexpr (GP) {
                         // the gen group wrote the chunk's gates (over its a tile, whose Z it has read)
-                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_GRDY + (c & 1)], (c >> 1) & 1, abort_flag, limit));
                         if (!ok) break;
                     } else {
                         if (c >= 2) {
-                            ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], ((c - 2) >> 1) & 1, abort_flag, kWaitLimitNs));
+                            ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], ((c - 2) >> 1) & 1, abort_flag, limit));
                             if (!ok) break;
                         }
-                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_FULL + c % kSlots], (c / kSlots) & 1, abort_flag, kWaitLimitNs));
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_FULL + c % kSlots], (c / kSlots) & 1, abort_flag, limit));
                         if (!ok) break;
                     }
                     tc_fence_after();
@@ -1038,15 +1038,14 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 auto full = [&](int c) -> uint64_t * { return &bars[BAR_GFULL + c % kSlots]; };
                 if constexpr (GP) {
                     for (int c = 0; c < 2 && c < G; ++c) {
-                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, kWaitLimitNs));
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c), 0, abort_flag, limit));
                         if (!ok) break;
                         tc_fence_after();
                         issue_z(c);
                     }
                 }
                 for (int c = 0; ok && c < G; ++c) {
-                    if (c == 2) wait_summaries();
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_PURDY + (c & 1)], (c >> 1) & 1, abort_flag, limit));
                     if (!ok) break;
                     tc_fence_after();
                     // GP: chunk c + 2's Z reuses the A buffer that gen(c) has read.  It goes before P(c) and
@@ -1083,7 +1082,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                     mma_commit2_warp(&bars[BAR_UFULL + (c & 1)], &bars[BAR_EMPTY + su]);  // U is the slot's last reader among this warp's MMAs
                     su = (su == kSlots - 1) ? 0 : su + 1;
                     if (z_due) {
-                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c + 2), ((c + 2) / kSlots) & 1, abort_flag, kWaitLimitNs));
+                        ok = !__any_sync(0xffffffffu, !mbar_wait(full(c + 2), ((c + 2) / kSlots) & 1, abort_flag, limit));
                         if (!ok) break;
                         tc_fence_after();
                         issue_z(c + 2);
@@ -1093,9 +1092,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 const uint32_t idesc_o = instr_desc(kFmtF16, 64, 64, 0, 1);
                 const uint32_t sbuf = smem_u32(smem + kOffS);
                 int so = 0;
-                wait_summaries();
                 for (int c = 0; c < G; ++c) {
-                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_ORDY + (c & 1)], (c >> 1) & 1, abort_flag, kWaitLimitNs));
+                    ok = !__any_sync(0xffffffffu, !mbar_wait(&bars[BAR_ORDY + (c & 1)], (c >> 1) & 1, abort_flag, limit));
                     if (!ok) break;
                     tc_fence_after();
                     // O(c) = Qtil S_[c] + P V  (fp16 mode: Q^ (Diag(c1) S_[c]) + P V); the key
@@ -1138,7 +1136,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         auto gen_out = [&](int co) {
             // (a lane whose wait gave up goes on with the others, as what follows is warp-collective; the group
             // leaves together at the barrier of its next chunk, and the outputs are then undefined)
-            if (!mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs)) record_timeout(abort_flag);
+            if (!mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, limit)) record_timeout(abort_flag);
             tc_fence_after();
             uint32_t r[32];
             tmem_ld_16x32bx2_x16(tmem + lane_base + kColO + (co & 1) * 64 + 0, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
@@ -1208,7 +1206,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             }
             // (a lane whose wait gave up goes on with the others, as the TMEM loads are warp-collective; the
             // group leaves together at the barrier of its next chunk)
-            if (!mbar_wait(&bars[BAR_ZFULL + zb], (cz >> 1) & 1, abort_flag, kWaitLimitNs)) record_timeout(abort_flag);
+            if (!mbar_wait(&bars[BAR_ZFULL + zb], (cz >> 1) & 1, abort_flag, limit)) record_timeout(abort_flag);
             tc_fence_after();
             uint8_t *gt = smem + kOffSlot + (cz % kSlots) * kSlotBytes + kG;
             uint32_t zr[32];
@@ -1238,9 +1236,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             const int sl = c % kSlots, bb = c & 1;
             const uint32_t ph = (c >> 1) & 1;
             uint8_t *st = smem + kOffSlot + sl * kSlotBytes;
-            bool fail = !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, kWaitLimitNs);
+            bool fail = !mbar_wait(&bars[BAR_AFULL + bb], ph, abort_flag, limit);
             // (gate producer: A(c) waited for the a tile only)
-            if constexpr (GP) fail = fail || !mbar_wait(&bars[BAR_FULL + sl], (c / kSlots) & 1, abort_flag, kWaitLimitNs);
+            if constexpr (GP) fail = fail || !mbar_wait(&bars[BAR_FULL + sl], (c / kSlots) & 1, abort_flag, limit);
             // bf16 values become fp16 MMA operands in place (exact for |v| in the fp16
             // normal range); the loads go first so that their latency hides behind the
             // operand build, the converted words are stored with the operands
@@ -1402,7 +1400,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             // ---- masked scores of chunk c over its gate tile (consumed by A(c) long ago)
             // (a warp that gives up here skips the rest of the chunk; the group leaves together at
             // the barrier of its next one)
-            const bool pfail = !mbar_wait(&bars[BAR_PFULL + bb], ph, abort_flag, kWaitLimitNs);
+            const bool pfail = !mbar_wait(&bars[BAR_PFULL + bb], ph, abort_flag, limit);
             if (__any_sync(0xffffffffu, pfail)) {
                 if (lane == 0) record_timeout(abort_flag);
                 continue;
@@ -1425,7 +1423,6 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[BAR_ORDY + bb]);  // this warp's rows of P are in smem
-            if (last_c < 0) wait_summaries();  // (after the group's first chunk)
             last_c = c;
         }
         if constexpr (kGenOut) {
@@ -1480,9 +1477,9 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
         // 16.4; B = 4, H = 12, 40 x 40 (3 segments of 9 chunks) the same 27.5.
         if constexpr (MODE == kSplitFull && NH == 1) {
             const int seg = pos(0).seg;
-            wait_summaries();  // the summaries are the previous grid's: this launch may start before it ends
             if (seg > 0) {
                 const StreamPos p0 = pos(0);
+                pdl_wait();  // the summaries are the previous grid's: this launch may start before it ends
                 const int te = threadIdx.x - 32 * kEpi0;
                 const int fr = te >> 4, fc = (te & 15) * 4;
                 float *ring = reinterpret_cast<float *>(smem + kOffSlot + 2 * kSlotBytes);  // 4 x [64][64]
@@ -1604,11 +1601,11 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         }  // (else: a split launch gives every CTA one segment, and S holds the fold)
                         dp = dpo = 1.f;
                     }
-                    bool fail = !mbar_wait(&bars[BAR_REFS + sl], (c / kSlots) & 1, abort_flag, kWaitLimitNs);
+                    bool fail = !mbar_wait(&bars[BAR_REFS + sl], (c / kSlots) & 1, abort_flag, limit);
                     // buffer bb was last read by O(c-2) (epi outputs with one key half: observed by
                     // the readout of the previous iteration already)
                     if (!kSum && (NH == 2 || kGenOut) && c >= 2)
-                        fail = fail || !mbar_wait(&bars[BAR_OFULL + bb], ph ^ 1, abort_flag, kWaitLimitNs);
+                        fail = fail || !mbar_wait(&bars[BAR_OFULL + bb], ph ^ 1, abort_flag, limit);
                     if (__any_sync(0xffffffffu, fail)) {  // the warp leaves together
                         ok = false;
                         break;
@@ -1631,7 +1628,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                         if (lane == 0) mbar_arrive(&bars[BAR_ORDY + bb]);  // with the outputs of c-2 read out
                     }
                     // state carry: S_[c+1] = Diag(d_c) S_[c] + Diag(c2) U_c
-                    fail = !mbar_wait(&bars[BAR_UFULL + bb], ph, abort_flag, kWaitLimitNs);
+                    fail = !mbar_wait(&bars[BAR_UFULL + bb], ph, abort_flag, limit);
                     if (__any_sync(0xffffffffu, fail)) {
                         ok = false;
                         break;
@@ -1701,7 +1698,7 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
                 if (!kSum && !kGenOut && c >= nh && c % nh == 0) {
                     // outputs of the real chunk whose last key half is c-1
                     const int co = c - 1, ob = (co / nh) & 1;
-                    const bool fail = !mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, kWaitLimitNs);
+                    const bool fail = !mbar_wait(&bars[BAR_OFULL + (co & 1)], (co >> 1) & 1, abort_flag, limit);
                     if (__any_sync(0xffffffffu, fail)) {
                         ok = false;
                         break;
@@ -1750,10 +1747,10 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
 
 // Test hook: launched between a split's passes, it stands for a summary pass that takes longer than the
 // limit of the bounded waits: the output pass starts while it runs and waits for it.
-__global__ void slow_grid_kernel() {
+__global__ void slow_grid_kernel(unsigned long long ns) {
     pdl_launch_dependents();
     const uint64_t t0 = global_timer_ns();
-    while (global_timer_ns() - t0 < kWaitLimitNs + kWaitLimitNs / 2) __nanosleep(1000000);
+    while (global_timer_ns() - t0 < ns) __nanosleep(1000);
 }
 
 // ---------------------------------------------------------------- host side
@@ -2176,6 +2173,7 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.seg_len = sp.len;
     tp.fd_L = make_fastdiv(sp.len);
     tp.summary = static_cast<float *>(workspace);
+    tp.wait_limit = kWaitLimitNs + kSummaryChunkNs * static_cast<unsigned long long>(sp.len);
     tp.flags = nullptr;
     tp.epoch = 0;
     // test hooks: 1, the timeout path (no fault: the data of one chunk simply never arrives); 2, a slow
@@ -2196,7 +2194,7 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
         sum_ctas = grid.x;
         e = half ? launch_shape<__half, kSummary>(grid, tp, stream) : launch_shape<__nv_bfloat16, kSummary>(grid, tp, stream);
         if (e != cudaSuccess) return e;
-        if (drop != nullptr && drop[0] == '2') slow_grid_kernel<<<1, 32, 0, stream>>>();
+        if (drop != nullptr && drop[0] == '2') slow_grid_kernel<<<1, 32, 0, stream>>>(kWaitLimitNs + kSummaryChunkNs / 2 * sp.len);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     tp.nsu = nseg;
