@@ -108,7 +108,7 @@ struct SwProblem {
     int B, grid_h, grid_w, F;
     int dtype;                  // 0 f32, 1 f16, 2 bf16
 };
-// Grids the kernel takes (a tile's box spans the grid width plus the halo).
+// Grids the entry point takes (up to 254 columns).
 bool sswiglu_supported(const SwProblem &p);
 cudaError_t launch_sswiglu(const SwProblem &p, cudaStream_t stream);
 // Status word of the S-SwiGLU kernel's bounded wait (kStatusTimeout).

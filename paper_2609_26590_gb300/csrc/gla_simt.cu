@@ -29,9 +29,13 @@
 // is walked again with the outputs.  One launch and no workspace: calls under stream
 // capture, on several streams or with no scratch run the same way.
 //
+// Narrow values, few key channels and short sequences would leave most of the tiles
+// empty: whole sequences of those take the kernel of 16 columns a CTA (narrow_columns).
+//
 // Measured on a GB300 (graph replays, fp32, Dk = Dv = 64), against one CTA of 256 threads
 // per 16 columns walking whole sequences: 24 sequences of 1,600 tokens 63 us (440 before),
-// 2 of 256 tokens 14 us (43 before).
+// 2 of 256 tokens 14 us (43 before).  Up to 32 key channels the helper and compute roles
+// spill (36 to 60 bytes of stores a thread, up to 64 channels 4).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 

@@ -39,8 +39,8 @@
 // permutation lives in the load coordinates and in the addresses of the output stores.
 //
 // Warp roles (512 threads, one CTA per SM; four warps per SM sub-partition, so a
-// thread keeps 128 registers).  Few roles with small loops keep the hot code
-// inside the SM's instruction cache:
+// thread keeps 128 registers).  All roles share the SM's instruction cache, so few
+// roles with small loops:
 //   warp 0       TMA producer.
 //   warp 1       TMEM allocator and issuer of A(c) = L G.
 //   warps 2-5    gen warpgroup 0 (even chunks): reads A, builds the operands of its
@@ -517,9 +517,10 @@ __device__ __forceinline__ void store_row(const TcParams &p, const uint32_t (&ow
 // prefix a of the clamped gates (log2), then P[rho][sigma] = sum_i q k 2^{a_r,i - a_j,i} (j <= r)
 // without a split that could overflow.  For a key block J of 16 scan positions before the row's own,
 // 2^{a_r - a_j} = 2^{a_r - a_e} 2^{a_e - a_j} with e the block's last position: both factors are at most
-// 1, the second one is formed once per key (kb), the first once per row and block.  The row's own block
-// does the same with blocks of 4, and only keys in the row's own 4 take an exponential each: about 550
-// per row instead of 2,080 on average (GB300, 6,400 tokens with the gate producer and strong decays
+// 1, the second one is formed once per key (kb), the first for every eight keys of a row.  The row's own block
+// does the same with blocks of 4, and only keys in the row's own 4 take an exponential each: about 670
+// per row instead of 2,080 on average (128 for kb, 192 and 96 for the row's factors in earlier blocks of 16
+// and 4, 256 in its own 4; a block of 16 is done in two halves, each with the row's factors anew) (GB300, 6,400 tokens with the gate producer and strong decays
 // 2,065 -> 1,367 us; B = 4, H = 8, 48 x 40, all chunks exact, 265 -> 170 us).  Also Qtil = q 2^{a},
 // Kbar = k 2^{a_last - a}, and the chunk decay.  `as` holds two 64 x 64 fp32 arrays, a and kb, whose
 // rows' float4s are permuted so that a warp's 16 rows fall into different banks.  SUM (summary passes): no scores and no queries, the q and gate tiles stay as they are.
@@ -773,9 +774,8 @@ __global__ void __launch_bounds__(kThreads, 1) gla_tc_kernel(const __grid_consta
     // which takes that work off the epi's serial per-chunk chain.  The host selects it where
     // that was measured faster (fp16 launches of at most one wave); elsewhere the epi stores.
     constexpr bool kGenOut = GENOUT && NH == 1 && !kSum;
-    // The SM's instruction cache is shared by all roles, and the hot loops do not fit it (ncu: 9 % of
-    // its requests miss on B = 32, H = 12, 40 x 40, 35 % with the gate producer).  The fp16 operand
-    // build therefore runs as a loop over two halves of a thread's channels, each read from TMEM when
+    // The SM's instruction cache is shared by all roles (ncu: 4 % of its requests miss on B = 32, H = 12,
+    // 40 x 40 and at Dk = Dv = 128, 14 % with the gate producer).  The fp16 operand build therefore runs as a loop over two halves of a thread's channels, each read from TMEM when
     // its turn comes, where the epi stores the outputs (GB300, graph replays: 84.5 -> 82.3 us there,
     // Dk = Dv = 128 188 -> 185 us); unrolled it is faster where the gen warps store them (6,400 tokens,
     // tf32 scores: 155 us against 171).
@@ -2004,11 +2004,14 @@ int pad64(int d) { return (d + 63) / 64 * 64; }
 // launch still fits one wave (units x ceil(N / len) <= SMs).  The split's critical
 // path is the last segment: `len` chunks in each of the two passes, plus the fold
 // of the nseg - 1 earlier summaries into its start state, with several summaries'
-// loads in flight.  A graph-replayed sweep of every length on a GB300, with the fold
-// before the first chunk (batch-1 and small-batch shapes, 64 <= N <= 256 chunks), fitted
-// about 1.95 us per chunk of length against 0.13 us per segment, so the length
-// minimises 15 len + ceil(N / len), at least kMinSegChunks.  Sequences of at most
-// kMaxUnsplitChunks chunks stay whole (5 chunks: 11.4 us whole, 13.4 us split).
+// loads in flight.  A graph-replayed sweep of every length on a GB300, of an earlier
+// kernel with the fold before the first chunk (batch-1 and small-batch shapes, 64 <= N <= 256
+// chunks), fitted about 1.95 us per chunk of length against 0.13 us per segment, so the
+// length minimises 15 len + ceil(N / len), at least kMinSegChunks.  (With the present kernels
+// two chunks of both passes take 4.0 us and a fold of 12 summaries 2.7; the constants were
+// not fitted again.)  Sequences of at most kMaxUnsplitChunks chunks stay whole (6 chunks: 8.9
+// us split; 5 chunks: 9.4 us whole and 9.0 split in fp16, 10.0 and 9.4 in bf16, so the line
+// could lie one lower now; with the earlier kernels 11.4 and 13.4).
 // The last segment may be shorter than the others: its chunks past the sequence
 // load as zeros (no key, decay 1), so they leave the state unchanged, and their
 // outputs are not stored.
@@ -2236,8 +2239,10 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     // bf16, 384 units on 128 CTAs instead of 152 ran 3 % faster, the same at fp16)
     const int per_cta = (tp.n_units + n_sm - 1) / n_sm;
     const dim3 grid(static_cast<unsigned>((tp.n_units + per_cta - 1) / per_cta));
-    // outputs from the gen warpgroups: fp16 launches of at most one wave (measured on a GB300:
-    // +3 to +6 % there; with several units per CTA, or bf16, the epi storing them was faster)
+    // outputs from the gen warpgroups: fp16 launches of at most one wave (GB300, graph replays, stored by
+    // the epi / here: 6,400 tokens, B = 8, H = 16, strong decays 149.6 / 148.0 us, mild 106.4 / 104.4; 64 heads
+    // of 64 x 64 80.9 / 79.5; 12 heads, B = 12, 40 x 40 32.5 / 32.1; six heads of 24 x 16 9.25 / 8.88.  With
+    // several units per CTA, or bf16, the epi storing them was faster, measured with earlier kernels)
     const bool gen_out = half && tp.n_units <= n_sm;
     // The output pass of a split starts while its summary pass runs (its CTAs start once every summary
     // CTA has).  One key half: always; CTAs load and prepare their first chunks on SMs as they free up

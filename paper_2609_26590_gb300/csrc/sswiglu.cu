@@ -282,7 +282,7 @@ bool encode(CUtensorMap *m, const SwProblem &p, const void *base, int box_w, int
 }  // namespace
 
 bool sswiglu_supported(const SwProblem &p) {
-    // grids up to 254 columns (tiles as wide as the grid and its halo would fit a TMA box)
+    // grids up to 254 columns: the entry point's documented range (the column tiles would take any width)
     return p.grid_w + 2 <= 256 && tensor_map_encoder() != nullptr;
 }
 
