@@ -106,7 +106,10 @@ constexpr uint64_t kWaitLimitNs = 1000000000ull;  // bounded waits give up after
 // what the slowest ones (all scores exact) take
 constexpr uint64_t kSummaryChunkNs = 100000ull;
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kGateMinLog2 = -1.0e4f * 1.4426950408889634f;  // g < -1e4 acts as -1e4
+// Gates below this (log2) act as it: 2^-128 is 0 (flushed) as any smaller decay is, and a chunk's prefix stays
+// above -8,192, whose last bit of 2^-10 the decays of the keys after a channel's last zero gate keep.  (With
+// gates clamped at -1e4 a few zero gates a channel left the prefix 2^-5 and the outputs 4e-3 off.)
+constexpr float kGateMinLog2 = -128.0f;
 constexpr float kMaxRefF16 = 8.0f;        // fp16 score operands: factors within 2^{+-8}
 constexpr float kMaxRefTF32 = 100.0f;     // tf32 score operands: factors within 2^{+-100}
 
