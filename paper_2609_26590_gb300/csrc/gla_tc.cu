@@ -190,6 +190,7 @@ struct TcParams {
                                            // [Dk][Dv] and total decay [Dk], fp32
     int drop_load;                         // test hook: CTA 0 withholds its first chunk's load, so the
                                            // bounded waits run out and the call reports a timeout
+    unsigned long long out_row;            // elements per token of the output, H Dv (2^31 and more at 2^24 heads)
     unsigned long long wait_limit;         // kSplitFull, one key half: the bounded waits' limit in ns
     unsigned long long *flags;             // kBalanced: per CTA, == epoch once its hand-off state (in
                                            // summary, [64][64] fp32 per CTA) is written; cleared when read
@@ -499,7 +500,7 @@ __device__ __forceinline__ void store_row(const TcParams &p, const uint32_t (&ow
         const int other = __shfl_xor_sync(0xffffffffu, t, 1);
         const int t0 = odd ? other : t, t1 = odd ? t : other;
         const int col = col0 + 8 * odd;
-        const size_t ld = (size_t)p.H * p.Dv;  // (2^31 elements and more at 2^24 heads)
+        const size_t ld = p.out_row;
         E *base = static_cast<E *>(p.out) + ((size_t)b * p.T * p.H + h) * p.Dv + col;
 #pragma unroll
         for (int q = 0; q < 4; q += 2) {
@@ -2155,6 +2156,7 @@ cudaError_t launch_tc(const Problem &p, cudaStream_t stream, void *workspace, si
     tp.out = p.out;
     tp.final_state = p.final_state;
     tp.H = p.H;
+    tp.out_row = static_cast<unsigned long long>(p.H) * p.Dv;
     tp.grid_h = p.grid_h;
     tp.fd_H = make_fastdiv(p.H);
     tp.fd_gh = make_fastdiv(p.grid_h);
@@ -2304,6 +2306,7 @@ cudaError_t launch_tc_gate(const Problem &p, const GateSource &gs, cudaStream_t 
     tp.out = p.out;
     tp.final_state = p.final_state;
     tp.H = p.H;
+    tp.out_row = static_cast<unsigned long long>(p.H) * p.Dv;
     tp.grid_h = p.grid_h;
     tp.fd_H = make_fastdiv(p.H);
     tp.fd_gh = make_fastdiv(p.grid_h);
